@@ -109,9 +109,10 @@ typedef struct pstd_plan_s pstd_plan_t;
  * e^{-ik dx/2} / M of the symmetric-periodic extension of each axis, Table 1)
  * and rounds them once to FP32; allocates them and one scratch accumulator of
  * the pressure shape (ndim >= 2) on the device.  Routes per axis, by the
- * period M of its extension: the register-FFT passes for M in {2..1024
- * powers of two, 96, 192, 384, 768}; shared-memory Stockham FFT passes for
- * other M with prime factors 2, 3 and 5 only; for any other M, a dense
+ * period M of its extension: the folded passes on walled axes with M >= 16
+ * and a radix schedule (pstd_plan_opts.variant 6); the register-FFT passes for
+ * other M in {2..1024 powers of two, 96, 192, 384, 768}; shared-memory
+ * Stockham FFT passes for other M with prime factors 2, 3 and 5 only; for any other M, a dense
  * operator matrix when N_i <= 64, else a (skew-)circular convolution of
  * length M evaluated as a linear convolution through a circular FFT of
  * length M2 >= 2M - 1: of the 2^a 3^b 5^c lengths up to the next power of
@@ -134,10 +135,13 @@ int pstd_plan(const pstd_desc* desc, void* stream, pstd_plan_t** out);
  * registers per thread, more resident CTAs; the default for length 768 on
  * axes with many lines), variant 5 (lengths 256, 512) the same with the
  * tables read from global memory through L1 (neither registers nor shared
- * memory hold them; the default for lengths 256 and 512 on axes with many
- * lines, the 3-D sizes); variants 3, 4 and 5 serve walled (non-periodic)
- * axes only and fix N = L / 2 at compile time.  An unavailable variant gives
- * PSTD_EINVAL.
+ * memory hold them); variants 3, 4 and 5 serve walled (non-periodic) axes
+ * only and fix N = L / 2 at compile time.  Variant 6, the default of every
+ * walled axis with 2N >= 16 whose 2N factors into its radices (all 2^a 3^b 5^c
+ * up to N = 1024 but 625, many with 7, 11 or 13, and larger ones), transforms
+ * the symmetry-folded line (one half of the extension and of its spectrum);
+ * without options the register-FFT variants serve periodic axes and lengths
+ * below 16.  An unavailable variant gives PSTD_EINVAL.
  * seqs_per_cta: line pairs per CTA (a power of two). */
 typedef struct {
     int variant[3];
@@ -229,7 +233,8 @@ int pstd_step(pstd_plan_t* plan, float* p, float* const* u);
 
 /* `nsteps` >= 0 leapfrog steps in place.  The plan records one block of
  * steps in a CUDA graph per (p, u) pointer set on first use and replays it;
- * a tail shorter than the block is launched directly.
+ * a tail shorter than the block is launched directly.  A 1-D run on a
+ * compiled folded schedule is one kernel that loops over its steps.
  * Errors: PSTD_EINVAL, PSTD_ECUDA. */
 int pstd_run(pstd_plan_t* plan, float* p, float* const* u, int64_t nsteps);
 

@@ -1,0 +1,78 @@
+// pstd_fold_launch.cu -- kernel choice and launch of the folded passes.
+#include "pstd_fkernels.cuh"
+
+namespace pstd {
+
+const void* fold_any_misc_s();
+const void* fold_any_misc_c();
+#define DECL(U) const void* fold_unit_##U(int R, int A, int B, int P, bool strided, int mode);
+PSTD_FOLD_UNITS(DECL)
+#undef DECL
+
+const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) {
+    fixed = true;
+    if (!x.wide && (mode == FOLD_STEP || mode == FOLD_ORDER2 || mode == FOLD_LINE)) {
+#define TRY(U) \
+    if (const void* k = fold_unit_##U(x.R, x.A, x.B, x.P, strided, mode)) return k;
+        PSTD_FOLD_UNITS(TRY)
+#undef TRY
+    }
+    fixed = false;
+    if (mode == FOLD_LINE) return nullptr;
+    if (mode == FOLD_STEP) return fold_any_step(strided);
+    return strided ? fold_any_misc_s() : fold_any_misc_c();
+}
+
+cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cudaStream_t st) {
+    bool fixed = false;
+    const void* k = fold_kernel(a.ax, strided, a.mode, fixed);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(g.grid);
+    // the run-time form loops over its work, so it takes no more threads than
+    // it is compiled for
+    cfg.blockDim = dim3(fixed || g.threads < fold::kAnyThreads ? g.threads : fold::kAnyThreads);
+    cfg.dynamicSmemBytes = g.smem;
+    cfg.stream = st;
+    // passes of a step follow one another: a pass may start (and fetch its
+    // tables) while the previous one drains; it waits before touching fields
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.mode == FOLD_STEP || a.mode == FOLD_ORDER2 ? 1 : 0;
+    void* args[] = {(void*)&a};
+    return cudaLaunchKernelExC(&cfg, k, args);
+}
+
+bool fold_has_line(const FoldAxis& x) {
+    bool fixed = false;
+    return x.nlines == 1 && fold_kernel(x, false, FOLD_LINE, fixed) != nullptr;
+}
+cudaError_t fold_launch_line(const FoldArgs& a, int64_t nsteps, const FoldLaunch& g, cudaStream_t st) {
+    bool fixed = false;
+    const void* k = fold_kernel(a.ax, false, FOLD_LINE, fixed);
+    void* args[] = {(void*)&a, (void*)&nsteps};
+    return cudaLaunchKernel(k, dim3(1), dim3(g.threads), args, g.smem, st);
+}
+
+cudaError_t fold_set_smem(const FoldAxis& x, bool strided, int bytes) {
+    for (int mode : {(int)FOLD_STEP, (int)FOLD_ORDER2, (int)FOLD_GRAD_P}) {
+        bool fixed = false;
+        const void* k = fold_kernel(x, strided, mode, fixed);
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    if (fold_has_line(x)) {
+        bool fixed = false;
+        const cudaError_t e = cudaFuncSetAttribute(fold_kernel(x, false, FOLD_LINE, fixed),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    cudaFuncAttributes fa{};
+    const void* k = fold_any_persist();
+    cudaError_t e = cudaFuncGetAttributes(&fa, k);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes - (int)fa.sharedSizeBytes);
+}
+
+}  // namespace pstd

@@ -25,6 +25,8 @@
 #include "../../include/pstd.h"
 #include "pstd_cta.cuh"
 #include "pstd_energy.h"
+#include "pstd_fkernels.cuh"
+#include "pstd_foldplan.h"
 #include "pstd_gemm.h"
 #include "pstd_internal.h"
 #include "pstd_tc16.h"
@@ -86,6 +88,10 @@ cudaError_t w1024_persist_blocks(int L, int V, int threads, size_t smem, int* bl
 }  // namespace pstd
 
 using pstd::FftPlan;
+using pstd::FoldArgs;
+using pstd::FoldAxis;
+using pstd::FoldLaunch;
+using pstd::FoldPersistArgs;
 using pstd::GradArgs;
 using pstd::LineOp;
 using pstd::StepArgs;
@@ -106,6 +112,8 @@ constexpr int kConvMaxFft = 8192;    // largest power-of-two FFT of the convolut
 constexpr int kGraphSteps = 32;
 constexpr int kGraphCache = 4;
 constexpr size_t kSmemBudget = 100 * 1024;
+constexpr int kFold = 6;             // pstd_plan_opts.variant of the folded passes
+constexpr int kFoldMinLength = 16;   // shorter extensions: the one-lane register FFTs
 
 enum { OP_GRAD_P = 0, OP_GRAD_U = 1, OP_STEP_P = 2, OP_STEP_U = 3, OP_INIT_P = 4, OP_COUNT = 5 };
 
@@ -151,6 +159,14 @@ struct Axis {
     float* d_dense2 = nullptr;
     WAxis wax{};
     WLaunch wgeo{};
+    // folded passes (pstd_fold.cuh; wv == kFold, wl: lanes per pair)
+    FoldAxis fax{};
+    FoldLaunch fgeo{};
+    float2* d_ftab = nullptr;         // twiddles tw | tc | th
+    float2* d_fcoef = nullptr;        // step coefficients per bin
+    float* d_fgrad[OP_COUNT] = {};    // derivative multipliers per bin (GRAD_P, GRAD_U, INIT_P)
+    float* d_f2fold = nullptr;        // second-order multiplier per bin, on first use
+    bool fold() const { return wl > 0 && wv == kFold; }
     // BF16 three-way split form on tcgen05: the two operators' BF16 slices
     // (D1: N x lp, D2: lp x N) and their TMA tensor maps
     uint16_t* d_tc16[2] = {nullptr, nullptr};
@@ -684,6 +700,13 @@ int build_order2(pstd_plan_s* P, int i) {
     if (a.ok2) return PSTD_OK;
     const pstd_desc& d = P->desc;
     const double s2 = (d.c0 * d.dt) * (d.c0 * d.dt);
+    if (a.fold()) {
+        std::vector<float> f;
+        pstd::fold_order2_coef(a.fax, a.dx, s2, f);
+        const int rc = upload(f, &a.d_f2fold);
+        if (rc == PSTD_OK) a.ok2 = 1;
+        return rc;
+    }
     std::vector<std::complex<double>> f(a.L);
     for (int n = 0; n < a.L; ++n)
         f[n] = (coeff(a, n, 0, 1.0) * coeff(a, n, 1, 1.0) * (double)a.L * s2).real();
@@ -716,6 +739,169 @@ int build_order2(pstd_plan_s* P, int i) {
     a.ok2 = 1;
     return PSTD_OK;
 }
+
+// Folded passes of axis i (pstd_fold.cuh): geometry, tables and launch.  `os`
+// line pairs per CTA (-1: chosen here).
+int build_fold(pstd_plan_s* P, int i, const pstd::FoldChoice& ch, int os) {
+    Axis& a = P->ax[i];
+    const pstd_desc& d = P->desc;
+    pstd::FoldTables t;
+    FoldAxis& x = a.fax;
+    pstd::fold_axis(a.N, a.bcl == PSTD_DIRICHLET, a.bcr == PSTD_DIRICHLET, ch, x, t);
+    x.nlines = a.nlines;
+    x.inner = a.inner;
+    a.strided = a.inner > 1;
+    x.wide = (int64_t)(a.N + 1) * a.inner >= (int64_t)1 << 30;
+    auto tiles = [&](int p) -> int64_t {
+        if (!a.strided) return (a.nlines + 2 * p - 1) / (2 * p);
+        return (a.nlines / a.inner) * ((a.inner + 2 * p - 1) / (2 * p));
+    };
+    auto fits = [&](int p) {
+        x.P = p;
+        return pstd::fold::smem_bytes(x, a.strided) <= 200 * 1024;
+    };
+    int p = os;
+    if (p < 0) {
+        // A compiled schedule's PS / PC pairs where that leaves enough CTAs for
+        // the GPU (narrow schedules fill an SM with fewer: 64^3, 20 lanes per
+        // pair, 9.6 us per step with 8 pairs on 256 CTAs, 20.9 with one pair);
+        // else 2 pairs on strided axes (512^2: 9.5 us with 129 CTAs of 2 against
+        // 11.5 with 1, whose 8-byte rows use a quarter of each sector) and 1
+        // on contiguous ones (512^2 with 2: 15.5).  Run-time schedules take 8 or
+        // fewer, within their thread count.
+        const int fixed = a.strided ? ch.PS : ch.PC;
+        if (fixed && !x.wide) {
+            const int64_t enough = pstd::fold_lanes(x) <= 48 ? P->nsm / 2 : (a.strided ? P->nsm : 2 * P->nsm);
+            p = tiles(fixed) >= enough ? fixed : (a.strided ? 2 : 1);
+        } else {
+            p = 8;
+            while (p > 1 && (tiles(p) < 2 * P->nsm || !fits(p) ||
+                             pstd::fold_lanes(x) * p > pstd::fold::kAnyThreads)) p /= 2;
+        }
+    }
+    if (!fits(p) || (os > 0 && pstd::fold_lanes(x) * p > 1024)) return os > 0 ? PSTD_EINVAL : PSTD_EUNSUPPORTED;
+    x.P = p;
+    x.lgP = 0;
+    while ((1 << x.lgP) < p) ++x.lgP;
+    a.fgeo.grid = (unsigned)tiles(p);
+    a.fgeo.threads = pstd::fold_threads(x);
+    a.fgeo.smem = pstd::fold::smem_bytes(x, a.strided);
+    std::vector<float2> tab(t.tw);
+    tab.insert(tab.end(), t.tc.begin(), t.tc.end());
+    tab.insert(tab.end(), t.th.begin(), t.th.end());
+    int rc;
+    if ((rc = upload(tab, &a.d_ftab)) != PSTD_OK) return rc;
+    x.tw = a.d_ftab;
+    x.tc = x.tw + t.tw.size();
+    x.th = x.tc + t.tc.size();
+    std::vector<float2> cf;
+    pstd::fold_step_coef(x, a.dx, -d.dt / d.rho0, -d.dt * d.rho0 * d.c0 * d.c0, cf);
+    if ((rc = upload(cf, &a.d_fcoef)) != PSTD_OK) return rc;
+    const struct { int op; double scale; } g[3] = {
+        {OP_GRAD_P, 1.0}, {OP_GRAD_U, 1.0}, {OP_INIT_P, d.dt / (2.0 * d.rho0)}};
+    for (const auto& q : g) {
+        std::vector<float> f;
+        pstd::fold_grad_coef(x, a.dx, q.scale, f);
+        if ((rc = upload(f, &a.d_fgrad[q.op])) != PSTD_OK) return rc;
+    }
+    a.wl = pstd::fold_lanes(x);
+    a.wv = kFold;
+    return PSTD_OK;
+}
+
+// Dense operators of the split forms of axis i (pstd_plan_opts.form 1, 2, 3).
+int build_forms(pstd_plan_s* P, int i) {
+    Axis& a = P->ax[i];
+    const pstd_desc& d = P->desc;
+    int rc;
+    const double scales[OP_COUNT] = {1.0, 1.0, -d.dt / d.rho0, -d.dt * d.rho0 * d.c0 * d.c0,
+                                     d.dt / (2.0 * d.rho0)};
+    // tensor-core split form: the dense operators of the two derivatives
+    // (FP64-built, scales folded in) as TF32 hi + lo parts
+    if (P->opts.form == 2) {
+        if (a.N > 1024) return PSTD_EUNSUPPORTED;
+        auto tf32 = [](double x) {
+            float f = (float)x;
+            uint32_t u;
+            std::memcpy(&u, &f, 4);
+            u = (u + 0x1000u) & 0xFFFFE000u;     // round to 10 mantissa bits, ties away
+            std::memcpy(&f, &u, 4);
+            return f;
+        };
+        const std::vector<double> D1 = dense_operator64(a, 0, scales[OP_STEP_P]);   // N x lp
+        const std::vector<double> D2 = dense_operator64(a, 1, scales[OP_STEP_U]);   // lp x N
+        std::vector<float> all;
+        for (const auto* D : {&D1, &D2}) {
+            std::vector<float> hi(D->size()), lo(D->size());
+            for (size_t j = 0; j < D->size(); ++j) {
+                hi[j] = tf32((*D)[j]);
+                lo[j] = tf32((*D)[j] - (double)hi[j]);
+            }
+            all.insert(all.end(), hi.begin(), hi.end());
+            all.insert(all.end(), lo.begin(), lo.end());
+        }
+        if ((rc = upload(all, &a.d_tc)) != PSTD_OK) return rc;
+    }
+
+    // BF16 three-way split form: both dense operators (FP64-built, scales
+    // folded in) as exact BF16 slices with their tensor maps
+    if (P->opts.form == 3) {
+        if (a.N > 1024) return PSTD_EUNSUPPORTED;
+        const std::vector<double> D1 = dense_operator64(a, 0, scales[OP_STEP_P]);   // nu x lp
+        const std::vector<double> D2 = dense_operator64(a, 1, scales[OP_STEP_U]);   // lp x nu
+        const int dims[2][2] = {{a.nu, a.lp}, {a.lp, a.nu}};
+        for (int o = 0; o < 2; ++o) {
+            const int r = pstd::tc16_operator(o == 0 ? D1 : D2, dims[o][0], dims[o][1], &a.d_tc16[o]);
+            if (r != 0) return cuda_fail((cudaError_t)r, "BF16 operator slices");
+            a.tc16_MT[o] = (dims[o][0] + 127) / 128;
+            a.tc16_KC[o] = pstd::tc16_chunks(dims[o][1]);
+        }
+    }
+
+    // split-precision dense form
+    if (P->opts.form == 1) {
+        if (a.N > 1024) return PSTD_EUNSUPPORTED;
+        std::vector<uint4> h1, l1, h2, l2;
+        double s1, s2;
+        gemm_fragments(dense_operator64(a, 0, scales[OP_STEP_P]), a.N, a.lp, h1, l1, s1);
+        gemm_fragments(dense_operator64(a, 1, scales[OP_STEP_U]), a.lp, a.N, h2, l2, s2);
+        std::vector<uint4> all;
+        all.insert(all.end(), h1.begin(), h1.end());
+        all.insert(all.end(), l1.begin(), l1.end());
+        all.insert(all.end(), h2.begin(), h2.end());
+        all.insert(all.end(), l2.begin(), l2.end());
+        if ((rc = upload(all, &a.d_gemm)) != PSTD_OK) return rc;
+        pstd::GemmAxis& g = a.gax;
+        g.N = a.N;
+        g.lp = a.lp;
+        g.MT1 = (a.N + 15) / 16;
+        g.KT1 = (a.lp + 15) / 16;
+        g.MT2 = (a.lp + 15) / 16;
+        g.KT2 = (a.N + 15) / 16;
+        g.A1h = a.d_gemm;
+        g.A1l = g.A1h + h1.size();
+        g.A2h = g.A1l + l1.size();
+        g.A2l = g.A2h + h2.size();
+        g.s1 = (float)s1;
+        g.s2 = (float)s2;
+        g.nlines = a.nlines;
+        g.inner = a.inner;
+        // lines per CTA: fit shared memory, and shrink until the axis has at
+        // least one CTA per SM
+        int G = 64;
+        while (G > 8 && pstd::gemm_smem_bytes(G, g.KT1, g.KT2, a.N) > 200 * 1024) G /= 2;
+        auto ctas = [&](int gg) {
+            return a.inner == 1 ? (a.nlines + gg - 1) / gg : (a.nlines / a.inner) * ((a.inner + gg - 1) / gg);
+        };
+        while (G > 8 && ctas(G) < P->nsm) G /= 2;
+        g.G = G;
+        a.gsmem = pstd::gemm_smem_bytes(G, g.KT1, g.KT2, a.N);
+        if (a.inner == 1) a.ggrid = (unsigned)((a.nlines + G - 1) / G);
+        else a.ggrid = (unsigned)((a.nlines / a.inner) * ((a.inner + G - 1) / G));
+    }
+    return PSTD_OK;
+}
+
 
 int build_axis(pstd_plan_s* P, int i) {
     Axis& a = P->ax[i];
@@ -850,6 +1036,19 @@ int build_axis(pstd_plan_s* P, int i) {
     a.G = G;
     a.smem = pstd::cta_smem_bytes(G, FL, a.rs);
     if (a.smem > 227 * 1024) return PSTD_EUNSUPPORTED;
+
+    // folded passes: every walled axis whose length has a schedule, unless the
+    // caller asks for a register-FFT schedule
+    {
+        const int ov = P->opts.variant[i], os = P->opts.seqs_per_cta[i];
+        pstd::FoldChoice ch{};
+        const bool can = !a.periodic && !a.mid && a.L >= kFoldMinLength && pstd::fold_choose(a.L, ch);
+        if (ov == kFold && !can) return PSTD_EINVAL;
+        if (can && (ov == kFold || (ov < 0 && (os < 0 || pstd::wlanes(a.L) == 0)))) {
+            if (os == 0 || os > 256 || (os > 0 && (os & (os - 1)))) return PSTD_EINVAL;
+            return build_fold(P, i, ch, ov == kFold ? os : -1);
+        }
+    }
 
     // register-FFT passes where a schedule exists.  Measured on GB300 (512^2,
     // 256^3, 384^3): the latency schedules (8 or 12 elements per lane) beat
@@ -1005,89 +1204,6 @@ int build_axis(pstd_plan_s* P, int i) {
         a.wv = V;
     }
 
-    // tensor-core split form: the dense operators of the two derivatives
-    // (FP64-built, scales folded in) as TF32 hi + lo parts
-    if (P->opts.form == 2) {
-        if (a.N > 1024) return PSTD_EUNSUPPORTED;
-        auto tf32 = [](double x) {
-            float f = (float)x;
-            uint32_t u;
-            std::memcpy(&u, &f, 4);
-            u = (u + 0x1000u) & 0xFFFFE000u;     // round to 10 mantissa bits, ties away
-            std::memcpy(&f, &u, 4);
-            return f;
-        };
-        const std::vector<double> D1 = dense_operator64(a, 0, scales[OP_STEP_P]);   // N x lp
-        const std::vector<double> D2 = dense_operator64(a, 1, scales[OP_STEP_U]);   // lp x N
-        std::vector<float> all;
-        for (const auto* D : {&D1, &D2}) {
-            std::vector<float> hi(D->size()), lo(D->size());
-            for (size_t j = 0; j < D->size(); ++j) {
-                hi[j] = tf32((*D)[j]);
-                lo[j] = tf32((*D)[j] - (double)hi[j]);
-            }
-            all.insert(all.end(), hi.begin(), hi.end());
-            all.insert(all.end(), lo.begin(), lo.end());
-        }
-        if ((rc = upload(all, &a.d_tc)) != PSTD_OK) return rc;
-    }
-
-    // BF16 three-way split form: both dense operators (FP64-built, scales
-    // folded in) as exact BF16 slices with their tensor maps
-    if (P->opts.form == 3) {
-        if (a.N > 1024) return PSTD_EUNSUPPORTED;
-        const std::vector<double> D1 = dense_operator64(a, 0, scales[OP_STEP_P]);   // nu x lp
-        const std::vector<double> D2 = dense_operator64(a, 1, scales[OP_STEP_U]);   // lp x nu
-        const int dims[2][2] = {{a.nu, a.lp}, {a.lp, a.nu}};
-        for (int o = 0; o < 2; ++o) {
-            const int r = pstd::tc16_operator(o == 0 ? D1 : D2, dims[o][0], dims[o][1], &a.d_tc16[o]);
-            if (r != 0) return cuda_fail((cudaError_t)r, "BF16 operator slices");
-            a.tc16_MT[o] = (dims[o][0] + 127) / 128;
-            a.tc16_KC[o] = pstd::tc16_chunks(dims[o][1]);
-        }
-    }
-
-    // split-precision dense form
-    if (P->opts.form == 1) {
-        if (a.N > 1024) return PSTD_EUNSUPPORTED;
-        std::vector<uint4> h1, l1, h2, l2;
-        double s1, s2;
-        gemm_fragments(dense_operator64(a, 0, scales[OP_STEP_P]), a.N, a.lp, h1, l1, s1);
-        gemm_fragments(dense_operator64(a, 1, scales[OP_STEP_U]), a.lp, a.N, h2, l2, s2);
-        std::vector<uint4> all;
-        all.insert(all.end(), h1.begin(), h1.end());
-        all.insert(all.end(), l1.begin(), l1.end());
-        all.insert(all.end(), h2.begin(), h2.end());
-        all.insert(all.end(), l2.begin(), l2.end());
-        if ((rc = upload(all, &a.d_gemm)) != PSTD_OK) return rc;
-        pstd::GemmAxis& g = a.gax;
-        g.N = a.N;
-        g.lp = a.lp;
-        g.MT1 = (a.N + 15) / 16;
-        g.KT1 = (a.lp + 15) / 16;
-        g.MT2 = (a.lp + 15) / 16;
-        g.KT2 = (a.N + 15) / 16;
-        g.A1h = a.d_gemm;
-        g.A1l = g.A1h + h1.size();
-        g.A2h = g.A1l + l1.size();
-        g.A2l = g.A2h + h2.size();
-        g.s1 = (float)s1;
-        g.s2 = (float)s2;
-        g.nlines = a.nlines;
-        g.inner = a.inner;
-        // lines per CTA: fit shared memory, and shrink until the axis has at
-        // least one CTA per SM
-        int G = 64;
-        while (G > 8 && pstd::gemm_smem_bytes(G, g.KT1, g.KT2, a.N) > 200 * 1024) G /= 2;
-        auto ctas = [&](int gg) {
-            return a.inner == 1 ? (a.nlines + gg - 1) / gg : (a.nlines / a.inner) * ((a.inner + gg - 1) / gg);
-        };
-        while (G > 8 && ctas(G) < P->nsm) G /= 2;
-        g.G = G;
-        a.gsmem = pstd::gemm_smem_bytes(G, g.KT1, g.KT2, a.N);
-        if (a.inner == 1) a.ggrid = (unsigned)((a.nlines + G - 1) / G);
-        else a.ggrid = (unsigned)((a.nlines / a.inner) * ((a.inner + G - 1) / G));
-    }
     return PSTD_OK;
 }
 
@@ -1100,6 +1216,10 @@ void free_plan_memory(pstd_plan_s* P) {
         cudaFree(a.d_fUL);
         cudaFree(a.d_ph);
         cudaFree(a.d_tc);
+        cudaFree(a.d_ftab);
+        cudaFree(a.d_fcoef);
+        cudaFree(a.d_f2fold);
+        for (float* f : a.d_fgrad) cudaFree(f);
         cudaFree(a.d_f2);
         cudaFree(a.d_dense2);
         for (int o = 0; o < 2; ++o)
@@ -1251,6 +1371,19 @@ StepArgs step_args(pstd_plan_s* P, int a, float* p, float* const* u) {
     return s;
 }
 
+FoldArgs fold_step(pstd_plan_s* P, int a, float* p, float* const* u) {
+    Axis& A = P->ax[a];
+    FoldArgs f{};
+    f.ax = A.fax;
+    f.mode = pstd::FOLD_STEP;
+    f.coef = A.d_fcoef;
+    f.in = p;
+    f.u = u[a];
+    f.acc_in = (a == P->ndim - 1) ? p : P->d_S;
+    f.out = (a == 0) ? p : P->d_S;
+    return f;
+}
+
 int launch_step(pstd_plan_s* P, float* p, float* const* u, int64_t* launches) {
     for (int a = P->ndim - 1; a >= 0; --a) {
         Axis& A = P->ax[a];
@@ -1335,6 +1468,11 @@ int launch_step(pstd_plan_s* P, float* p, float* const* u, int64_t* launches) {
             ++*launches;
             continue;
         }
+        if (A.fold()) {
+            CK(pstd::fold_launch(fold_step(P, a, p, u), A.strided, A.fgeo, P->stream));
+            ++*launches;
+            continue;
+        }
         if (A.wl) {
             WStep w;
             w.ax = A.wax;
@@ -1358,6 +1496,17 @@ int launch_step(pstd_plan_s* P, float* p, float* const* u, int64_t* launches) {
 
 int launch_grad(pstd_plan_s* P, int axis, int opi, const float* in, float* out, int acc) {
     Axis& A = P->ax[axis];
+    if (A.fold()) {
+        FoldArgs f{};
+        f.ax = A.fax;
+        f.mode = A.op[opi].dir == 0 ? pstd::FOLD_GRAD_P : pstd::FOLD_GRAD_U;
+        f.f = A.d_fgrad[opi];
+        f.in = in;
+        f.out = out;
+        f.accumulate = acc;
+        CK(pstd::fold_launch(f, A.strided, A.fgeo, P->stream));
+        return PSTD_OK;
+    }
     if (A.wl) {
         WGrad g;
         g.ax = A.wax;
@@ -1388,6 +1537,18 @@ int launch_grad(pstd_plan_s* P, int axis, int opi, const float* in, float* out, 
 // axis, and pout = in + out (the new value) where pout is given.
 int launch_order2(pstd_plan_s* P, int axis, const float* in, float* out, float* pout) {
     Axis& A = P->ax[axis];
+    if (A.fold()) {
+        FoldArgs f{};
+        f.ax = A.fax;
+        f.mode = pstd::FOLD_ORDER2;
+        f.f = A.d_f2fold;
+        f.in = in;
+        f.out = out;
+        f.accumulate = 1;
+        f.pout = pout;
+        CK(pstd::fold_launch(f, A.strided, A.fgeo, P->stream));
+        return PSTD_OK;
+    }
     if (A.wl) {
         WGrad g{};
         g.ax = A.wax;
@@ -1484,6 +1645,17 @@ int convert_velocity(pstd_plan_s* P, float* const* u, int dir, int64_t* launches
     for (int a = 0; a < P->ndim; ++a) {
         Axis& A = P->ax[a];
         if (!A.wl) continue;
+        if (A.fold()) {
+            FoldArgs f{};
+            f.ax = A.fax;
+            f.mode = dir == 2 ? pstd::FOLD_TO_SPEC : pstd::FOLD_FROM_SPEC;
+            f.in = u[a];
+            f.u = u[a];
+            f.out = u[a];
+            CK(pstd::fold_launch(f, A.strided, A.fgeo, P->stream));
+            ++*launches;
+            continue;
+        }
         WGrad g;
         g.ax = A.wax;
         g.dir = dir;
@@ -1513,6 +1685,17 @@ int pstd_internal_launch_steps(pstd_plan_t* P, float* p, float* const* u, int64_
     return PSTD_OK;
 }
 
+// Barrier of a cooperative run on the words count, generation, status at `d`.
+static GridSync grid_barrier(unsigned* d, unsigned grid, unsigned withhold, long long spin_limit) {
+    GridSync s;
+    s.count = d;
+    s.gen = d + 1;
+    s.status = (int*)(d + 2);
+    s.expected = grid + withhold;
+    s.spin_limit = spin_limit > 0 ? spin_limit : 2000000LL;   // ~0.2-1 s of polls
+    return s;
+}
+
 // ---- batch of plans as one cooperative kernel ------------------------------
 struct pstd_batch_persist_s {
     std::vector<unsigned char> h_args;   // WStep or StepArgs, [members][3]
@@ -1532,7 +1715,8 @@ int pstd_internal_batch_persist_kind(pstd_plan_t* const* plans, int n) {
     for (int m = 0; m < n && reg; ++m)
         for (int a = 0; a < plans[m]->ndim && reg; ++a) {
             const Axis& A = plans[m]->ax[a];
-            reg = A.wl > 0 && A0.wl > 0 && A.L == A0.L && A.wv == A0.wv && A.wgeo.threads == A0.wgeo.threads;
+            reg = A.wl > 0 && A0.wl > 0 && A.L == A0.L && A.wv == A0.wv &&
+                  (A.fold() || A.wgeo.threads == A0.wgeo.threads);
         }
     return reg ? 1 : 2;
 }
@@ -1570,7 +1754,9 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
     pstd_batch_persist_s* S = *state;
     int npass = 0;
     for (int m = 0; m < n; ++m) npass = plans[m]->ndim > npass ? plans[m]->ndim : npass;
-    const size_t esz = kind == 1 ? sizeof(WStep) : sizeof(StepArgs);
+    const bool fold = kind == 1 && plans[0]->ax[0].fold();
+    int fold_threads = 0;
+    const size_t esz = fold ? sizeof(FoldArgs) : (kind == 1 ? sizeof(WStep) : sizeof(StepArgs));
     S->h_args.assign((size_t)n * 3 * esz, 0);
     S->h_prefix.assign((size_t)3 * (n + 1), 0);
     size_t smem = 0;
@@ -1584,7 +1770,13 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
             if (a >= 0) {
                 Axis& A = P->ax[a];
                 unsigned char* slot = S->h_args.data() + ((size_t)m * 3 + k) * esz;
-                if (kind == 1) {
+                if (fold) {
+                    const FoldArgs f = fold_step(P, a, p[m], u + 3 * m);
+                    std::memcpy(slot, &f, sizeof f);
+                    items = A.fgeo.grid;
+                    smem = A.fgeo.smem > smem ? A.fgeo.smem : smem;
+                    fold_threads = A.fgeo.threads > fold_threads ? A.fgeo.threads : fold_threads;
+                } else if (kind == 1) {
                     WStep w;
                     w.ax = A.wax;
                     w.fP = A.d_f[OP_STEP_P];
@@ -1630,7 +1822,10 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const Axis& A0 = plans[0]->ax[0];
-    if (kind == 1) CK(wpersist_blocks(A0.L, A0.wv, A0.wgeo.threads, smem, &per_sm));
+    if (fold) {
+        if (fold_threads > pstd::fold::kAnyThreads) fold_threads = pstd::fold::kAnyThreads;
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pstd::fold_any_persist(), fold_threads, smem));
+    } else if (kind == 1) CK(wpersist_blocks(A0.L, A0.wv, A0.wgeo.threads, smem, &per_sm));
     else {
         CK(pstd::set_max_smem((int)smem));
         CK(pstd::k_step_persist_blocks(smem, &per_sm));
@@ -1639,13 +1834,19 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
     int64_t grid = (int64_t)per_sm * nsm;
     if (grid > most) grid = most;
     if (grid < 1) grid = 1;
-    GridSync sync;
-    sync.count = S->d_sync;
-    sync.gen = S->d_sync + 1;
-    sync.status = (int*)(S->d_sync + 2);
-    sync.expected = (unsigned)grid + withhold;
-    sync.spin_limit = spin_limit > 0 ? spin_limit : 2000000LL;
-    if (kind == 1) {
+    const GridSync sync = grid_barrier(S->d_sync, (unsigned)grid, withhold, spin_limit);
+    if (fold) {
+        FoldPersistArgs pa{};
+        pa.ndim = npass;
+        pa.nsteps = nsteps;
+        pa.sync = sync;
+        pa.members = n;
+        pa.mem = (const FoldArgs*)S->d_args;
+        pa.prefix = S->d_prefix;
+        void* args[] = {(void*)&pa};
+        CK(cudaLaunchCooperativeKernel(pstd::fold_any_persist(), dim3((unsigned)grid), dim3(fold_threads), args, smem,
+                                       st));
+    } else if (kind == 1) {
         PersistArgs pa{};
         pa.ndim = npass;
         pa.nsteps = nsteps;
@@ -1723,8 +1924,8 @@ int pstd_plan_schedule(const pstd_plan_t* P, int axis, int out[4]) {
     }
     out[0] = A.wv;
     out[1] = A.wl;
-    out[2] = A.wax.seqs;
-    out[3] = (int)A.wgeo.grid;
+    out[2] = A.fold() ? A.fax.P : A.wax.seqs;
+    out[3] = (int)(A.fold() ? A.fgeo.grid : A.wgeo.grid);
     return PSTD_OK;
 }
 
@@ -1764,7 +1965,10 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
         // velocity half-nodes; N - 1 next to a Neumann mid-cell wall
         P->shape[f][f - 1] = desc->ncells[f - 1] - (desc->bc[f - 1][1] == PSTD_NEUMANN_MID ? 1 : 0);
     }
-    for (int i = 0; i < P->ndim && rc == PSTD_OK; ++i) rc = build_axis(P, i);
+    for (int i = 0; i < P->ndim && rc == PSTD_OK; ++i) {
+        rc = build_axis(P, i);
+        if (rc == PSTD_OK && P->opts.form != 0) rc = build_forms(P, i);
+    }
     if (rc == PSTD_OK && P->opts.form == 3) rc = tc16_setup(P);
     if (rc == PSTD_OK && (P->opts.form == 2 || P->opts.form == 3)) {
         // status word of the tensor-core GEMMs' bounded waits (read by pstd_sync)
@@ -1797,7 +2001,8 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
             int dev = 0, optin = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-            e = wsmem(P->ax[i].L, P->ax[i].wv, optin);
+            e = P->ax[i].fold() ? pstd::fold_set_smem(P->ax[i].fax, P->ax[i].strided, optin)
+                                : wsmem(P->ax[i].L, P->ax[i].wv, optin);
             if (e != cudaSuccess) rc = cuda_fail(e, "cudaFuncSetAttribute(register-FFT pass)");
         }
     }
@@ -1806,19 +2011,29 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
         bool same = P->opts.form == 0;
         for (int i = 0; i < P->ndim && same; ++i)
             same = P->ax[i].wl > 0 && P->ax[i].L == P->ax[0].L && P->ax[i].wv == P->ax[0].wv &&
-                   P->ax[i].wgeo.threads == P->ax[0].wgeo.threads;
+                   (P->ax[i].fold() ? P->ax[i].fax.R == P->ax[0].fax.R && P->ax[i].fax.A == P->ax[0].fax.A
+                                    : P->ax[i].wgeo.threads == P->ax[0].wgeo.threads);
         if (same) {
+            const bool fold = P->ax[0].fold();
             size_t smem = 0;
             int64_t items = 0;
+            int threads = 0;
             for (int i = 0; i < P->ndim; ++i) {
-                smem = P->ax[i].wgeo.smem > smem ? P->ax[i].wgeo.smem : smem;
-                items = (int64_t)P->ax[i].wgeo.grid > items ? (int64_t)P->ax[i].wgeo.grid : items;
+                const size_t sm = fold ? P->ax[i].fgeo.smem : P->ax[i].wgeo.smem;
+                const int64_t it = fold ? P->ax[i].fgeo.grid : P->ax[i].wgeo.grid;
+                const int th = fold ? P->ax[i].fgeo.threads : P->ax[i].wgeo.threads;
+                smem = sm > smem ? sm : smem;
+                items = it > items ? it : items;
+                threads = th > threads ? th : threads;
             }
+            if (fold && threads > pstd::fold::kAnyThreads) threads = pstd::fold::kAnyThreads;
             int per_sm = 0, dev = 0, nsm = 0;
             cudaError_t e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
             if (e == cudaSuccess)
-                e = wpersist_blocks(P->ax[0].L, P->ax[0].wv, P->ax[0].wgeo.threads, smem, &per_sm);
+                e = fold ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pstd::fold_any_persist(), threads,
+                                                                         smem)
+                         : wpersist_blocks(P->ax[0].L, P->ax[0].wv, threads, smem, &per_sm);
             if (e == cudaSuccess) e = cudaMalloc((void**)&P->d_sync, 4 * sizeof(unsigned));
             if (e == cudaSuccess) e = cudaMemset(P->d_sync, 0, 4 * sizeof(unsigned));
             if (e != cudaSuccess) rc = cuda_fail(e, "persistent set-up");
@@ -1826,7 +2041,7 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
                 int64_t grid = (int64_t)per_sm * nsm;
                 if (grid > items) grid = items;
                 P->pgeo.grid = (unsigned)grid;
-                P->pgeo.threads = P->ax[0].wgeo.threads;
+                P->pgeo.threads = threads;
                 P->pgeo.smem = smem;
                 P->persist_ok = 1;
             }
@@ -1952,6 +2167,25 @@ int pstd_run(pstd_plan_t* P, float* p, float* const* u, int64_t nsteps) {
 namespace {
 // The steps of pstd_run with every register-FFT velocity in spectrum form.
 int run_steps(pstd_plan_t* P, float* p, float* const* u, int64_t nsteps) {
+    if (P->persist_ok && nsteps > 0 && P->ax[0].fold()) {
+        FoldPersistArgs pa{};
+        pa.ndim = P->ndim;
+        pa.nsteps = nsteps;
+        for (int a = 0; a < P->ndim; ++a) {
+            pa.ax[a] = fold_step(P, a, p, u);
+            pa.strided[a] = P->ax[a].strided ? 1 : 0;
+            pa.items[a] = P->ax[a].fgeo.grid;
+        }
+        pa.sync = grid_barrier(P->d_sync, P->pgeo.grid,
+                               (unsigned)(P->opts.withhold_arrivals > 0 ? P->opts.withhold_arrivals : 0),
+                               P->opts.spin_limit);
+        CK(cudaMemsetAsync(P->d_sync, 0, sizeof(unsigned), P->stream));   // arrival count
+        void* args[] = {(void*)&pa};
+        CK(cudaLaunchCooperativeKernel(pstd::fold_any_persist(), dim3(P->pgeo.grid), dim3(P->pgeo.threads), args,
+                                       P->pgeo.smem, P->stream));
+        P->last_launches = 1;
+        return PSTD_OK;
+    }
     if (P->persist_ok && nsteps > 0) {
         PersistArgs pa{};
         pa.ndim = P->ndim;
@@ -1969,13 +2203,16 @@ int run_steps(pstd_plan_t* P, float* p, float* const* u, int64_t nsteps) {
             pa.strided[a] = A.strided ? 1 : 0;
             pa.items[a] = A.wgeo.grid;
         }
-        pa.sync.count = P->d_sync;
-        pa.sync.gen = P->d_sync + 1;
-        pa.sync.status = (int*)(P->d_sync + 2);
-        pa.sync.expected = P->pgeo.grid + (unsigned)(P->opts.withhold_arrivals > 0 ? P->opts.withhold_arrivals : 0);
-        pa.sync.spin_limit = P->opts.spin_limit > 0 ? P->opts.spin_limit : 2000000LL;   // ~0.2-1 s of polls
+        pa.sync = grid_barrier(P->d_sync, P->pgeo.grid,
+                               (unsigned)(P->opts.withhold_arrivals > 0 ? P->opts.withhold_arrivals : 0),
+                               P->opts.spin_limit);
         CK(cudaMemsetAsync(P->d_sync, 0, sizeof(unsigned), P->stream));   // arrival count
         CK(wpersist(P->ax[0].L, P->ax[0].wv, P->pgeo, P->stream, pa));
+        P->last_launches = 1;
+        return PSTD_OK;
+    }
+    if (P->ndim == 1 && P->opts.form == 0 && P->ax[0].fold() && P->ax[0].fax.P == 1 && pstd::fold_has_line(P->ax[0].fax)) {
+        CK(pstd::fold_launch_line(fold_step(P, 0, p, u), nsteps, P->ax[0].fgeo, P->stream));
         P->last_launches = 1;
         return PSTD_OK;
     }

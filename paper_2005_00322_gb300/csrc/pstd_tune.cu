@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/pstd.h"
+#include "pstd_foldplan.h"
 #include "pstd_wkernels.cuh"
 
 namespace {
@@ -122,6 +123,21 @@ extern "C" int pstd_plan_autotune(const pstd_desc* desc, void* stream, const pst
     }
     for (int a = 0; a < desc->ndim && rc == PSTD_OK; ++a) {
         const int L = fft_length(desc, a);
+        // the compiled pairs per CTA of the folded passes
+        pstd::FoldChoice ch{};
+        if (desc->bc[a][0] != PSTD_PERIODIC && L >= 16 && pstd::fold_choose(L, ch) && ch.PS > 0) {
+            const bool strided = a + 1 < desc->ndim;
+            for (int sq : {strided ? ch.PS : ch.PC, strided ? 2 : 1}) {
+                pstd_plan_opts c = best.opts;
+                c.variant[a] = 6;
+                c.seqs_per_cta[a] = sq;
+                const double us = time_step(desc, c, st, f[0], f.data() + 1);
+                if (us > 0 && us < 0.98 * best.us) {
+                    best.us = us;
+                    best.opts = c;
+                }
+            }
+        }
         if (L <= 0 || pstd::wlanes(L) == 0) continue;
         const int lanes[6] = {pstd::wlanes(L), pstd::wlanes_latency(L), pstd::wlanes_v2(L), pstd::wlanes_v3(L),
                               pstd::wlanes_v4(L), pstd::wlanes_v5(L)};
