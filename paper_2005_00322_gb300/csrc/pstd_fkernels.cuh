@@ -108,6 +108,21 @@ const void* fold_fixed(int P, bool strided, int mode) {
         return nullptr;                                                                \
     }
 
+// Convolution pass on an embedding's radices (2 pairs per CTA strided, 1
+// contiguous), or null.
+template <int R, int A, int B>
+const void* conv_fixed(bool strided) {
+    return strided ? (const void*)fold::k_fold<fold::Cfg<R, A, B, 2>, true, FOLD_CONV>
+                   : (const void*)fold::k_fold<fold::Cfg<R, A, B, 1>, false, FOLD_CONV>;
+}
+#define PSTD_CONV_CASE(RR, AA, BB) \
+    if (R == RR && A == AA && B == BB) return conv_fixed<RR, AA, BB>(strided);
+#define PSTD_CONV_UNIT(U)                                                \
+    const void* conv_unit_##U(int R, int A, int B, bool strided) {       \
+        PSTD_CONV_U##U(PSTD_CONV_CASE)                                   \
+        return nullptr;                                                  \
+    }
+
 // pstd_fold_any*.cu: the run-time schedules.  mode < 0: one kernel for the
 // derivative, conversion and second-order modes.
 const void* fold_any_step(bool strided);

@@ -31,6 +31,14 @@
 // bookkeeping: N real coefficients per line, stored in the velocity's own
 // buffer (slot b - 1 for NN walls, whose bin 0 vanishes, else slot b).
 //
+// A line of any other length N (convolution passes, cN = N below) is embedded:
+// the derivative is the convolution of the extension with an odd kernel at
+// half-integer lags, and N half-node outputs of the nodes |j| <= N (or the
+// reverse) only need its lags |t| < 2N.  Cutting the kernel off there and laying
+// both on a circle of L = 2 N' >= 4N positions keeps every symmetry (even or
+// odd about 0, hence also about N'), so each derivative is a folded transform
+// of length L with zeros beyond N, a real multiplier and a folded inverse.
+//
 // A pass runs as five phases with a CTA barrier between them, in place in one
 // shared-memory buffer (element (r, k1, t) of the first radix, (r, k = k1 + A k2)
 // of the second and (r, k) of the combination share addresses):
@@ -55,6 +63,7 @@ struct FoldAxis {
     int wide;                // a CTA's lines span 4 GiB or more: 64-bit offsets
     int nk;                  // butterflies: pairs {k, M - g - k}
     int s0;                  // velocity slot of bin b is b - s0
+    int cN;                  // convolution passes: cells of the line (N = L / 2 is the embedding's); else 0
     float sg, rho;           // sign of p reflected about the left / right wall
     const float2* tw;        // [k1][t] exp(-i pi t (2 k1 + g) / M), A B entries
     const float2* tc;        // [r - 1][k] exp(-i pi r (2k + g) / L), r = 1..R/2
@@ -63,13 +72,15 @@ struct FoldAxis {
 };
 
 enum { FOLD_STEP = 0, FOLD_GRAD_P = 1, FOLD_GRAD_U = 2, FOLD_TO_SPEC = 3, FOLD_FROM_SPEC = 4, FOLD_ORDER2 = 5,
+       FOLD_CONV = 7,        // leapfrog pass of an embedded line: p -> u, u += , u -> p, p +=
        FOLD_LINE = 6 };        // FOLD_LINE: the kernel that loops over FOLD_STEP passes of a 1-D run
 
 struct FoldArgs {
     FoldAxis ax;
     int mode;
     const float2* coef;      // FOLD_STEP: per bin b <= N (p -> V, V -> p); zero where a bin has no slot
-    const float* f;          // FOLD_GRAD_*, FOLD_ORDER2: per bin multiplier (without the factor i)
+    const float* f;          // FOLD_GRAD_*, FOLD_ORDER2, FOLD_CONV p -> u: per bin multiplier (without the factor i)
+    const float* f2;         // FOLD_CONV u -> p
     const float* in;         // p (STEP, GRAD_P, ORDER2) or u
     float* u;                // velocity spectrum (STEP, TO_SPEC, FROM_SPEC)
     const float* acc_in;     // STEP: out = acc_in + contribution (contiguous axes: acc_in == in)
@@ -355,8 +366,8 @@ struct Pass {
     // the velocity slots after p1 (contiguous: before it), the accumulator
     // after p3.  A contiguous leapfrog pass accumulates onto p itself, which
     // p5's thread has read in p1; the second-order pass keeps that p for pout.
-    static constexpr bool ahead = C::fixed && (MODE == FOLD_STEP || MODE == FOLD_ORDER2);
-    static constexpr bool ahead_u = ahead && MODE == FOLD_STEP;
+    static constexpr bool ahead = C::fixed && (MODE == FOLD_STEP || MODE == FOLD_ORDER2 || MODE == FOLD_CONV);
+    static constexpr bool ahead_u = C::fixed && MODE == FOLD_STEP;
     static constexpr bool onto_p = ahead_u && !STR;
     static constexpr bool keep_p = ahead && MODE == FOLD_ORDER2 && STR;
     float2 uw[ahead_u ? C::R : 1];
@@ -373,11 +384,24 @@ struct Pass {
     PSTD_HD int Ap() const { return padded(A()); }
     PSTD_HD int S1() const { return Ap() * B(); }
     PSTD_HD int NRmax() const { return R() / 2 + 1; }
-    PSTD_HD int mode() const { if constexpr (MODE >= 0) return MODE; else return a.mode; }
-    PSTD_HD bool in_half() const { return mode() == FOLD_GRAD_U || mode() == FOLD_TO_SPEC; }
-    PSTD_HD bool out_half() const { return mode() == FOLD_GRAD_P || mode() == FOLD_FROM_SPEC; }
-    PSTD_HD int nin() const { return in_half() ? N() : a.ax.lp; }
-    PSTD_HD int nout() const { return out_half() ? N() : a.ax.lp; }
+    // PM: the mode a phase runs in; a convolution pass runs a FOLD_GRAD_P and a
+    // FOLD_GRAD_U
+    template <int PM = MODE>
+    PSTD_HD int mode() const { if constexpr (PM >= 0) return PM; else return a.mode; }
+    template <int PM = MODE>
+    PSTD_HD bool in_half() const { return mode<PM>() == FOLD_GRAD_U || mode<PM>() == FOLD_TO_SPEC; }
+    template <int PM = MODE>
+    PSTD_HD bool out_half() const { return mode<PM>() == FOLD_GRAD_P || mode<PM>() == FOLD_FROM_SPEC; }
+    PSTD_HD bool conv() const {
+        if constexpr (MODE == FOLD_CONV) return true;
+        else if constexpr (MODE >= 0) return false;
+        else return a.ax.cN > 0;
+    }
+    PSTD_HD int nhalf() const { return conv() ? a.ax.cN : N(); }     // stored half-nodes
+    template <int PM = MODE>
+    PSTD_HD int nin() const { return in_half<PM>() ? nhalf() : a.ax.lp; }
+    template <int PM = MODE>
+    PSTD_HD int nout() const { return out_half<PM>() ? nhalf() : a.ax.lp; }
 
     // f(pair p, work w) for this thread's items of W per pair
     template <class F>
@@ -453,14 +477,15 @@ struct Pass {
     // wall beyond it) or half-node j.  For even A the positions below e = A/2
     // lie before the right wall, so which elements are reflected is known at
     // compile time, and only node 0 and node N may be absent.
+    template <int PM = MODE>
     PSTD_HD void p1() {
-        if (mode() == FOLD_FROM_SPEC) return;
+        if (mode<PM>() == FOLD_FROM_SPEC) return;
         by_full([&](auto full) {
         with_radix<C::A>(A(), [&](auto RA) {
             constexpr int a_ = decltype(RA)::value;
             constexpr bool even = a_ % 2 == 0;
-            const bool half = in_half();
-            const int n = N(), lo = half ? 0 : a.ax.lo, len = nin();
+            const bool half = in_half<PM>();
+            const int n = N(), lo = half ? 0 : a.ax.lo, len = nin<PM>();
             const int refl = half ? 2 * n - 1 : 2 * n;   // position j reflects to refl - j
             const float rsg = half ? -a.ax.rho : a.ax.rho;
             const float* xa = base(a.in, len);
@@ -480,11 +505,11 @@ struct Pass {
                     const bool mir = even ? 2 * e >= a_ : (half ? j >= n : j > n);
                     const Off off = mir ? om - (Off)e * step : od + (Off)e * step;
                     bool ok = true;
-                    if (!half && (!even || e == 0 || 2 * e == a_)) {
-                        const int i = (mir ? refl - j : j) - lo;
-                        ok = i >= 0 && i < len;
-                    }
+                    const int i = (mir ? refl - j : j) - lo;
+                    if (conv() || (!half && (!even || e == 0 || 2 * e == a_))) ok = i >= 0 && i < len;
                     x[e] = make_float2(ok && la ? ld(xa, off) : 0.0f, ok && lb ? ld(xb, off) : 0.0f);
+                    // node N of an embedded line stands at both ends of its window
+                    if (conv() && !half && i + lo == a.ax.cN) x[e] = cscale(x[e], 0.5f);
                     if constexpr (onto_p) ac[e] = x[e];
                     if constexpr (keep_p) pk[e] = x[e];
                     if (mir) x[e] = cscale(x[e], rsg);
@@ -520,13 +545,15 @@ struct Pass {
             }
         });
     }
+    template <int PM = MODE>
     PSTD_HD void p2() {
-        if (mode() == FOLD_FROM_SPEC) return;
-        inner_radix<false>(in_half() ? R() / 2 : R() / 2 + 1);
+        if (mode<PM>() == FOLD_FROM_SPEC) return;
+        inner_radix<false>(in_half<PM>() ? R() / 2 : R() / 2 + 1);
     }
+    template <int PM = MODE>
     PSTD_HD void p4() {
-        if (mode() == FOLD_TO_SPEC) return;
-        inner_radix<true>(out_half() ? R() / 2 : R() / 2 + 1);
+        if (mode<PM>() == FOLD_TO_SPEC) return;
+        inner_radix<true>(out_half<PM>() ? R() / 2 : R() / 2 + 1);
     }
 
     // velocity slots of pair p: x = the spectrum's real part, y = its
@@ -586,6 +613,7 @@ struct Pass {
     }
 
     // p3: butterfly k of pair p: radix R, spectral update, radix R
+    template <int PM = MODE>
     PSTD_HD void p3() {
         with_even<C::R>(R(), [&](auto RR) {
             constexpr int r_ = decltype(RR)::value;
@@ -598,8 +626,8 @@ struct Pass {
                 const int rs = STR ? S1() * P() : S1();   // next residue
                 float2* s = at(0, p);
                 float2 w[r_];
-                if (mode() != FOLD_FROM_SPEC) {
-                    if (in_half()) {
+                if (mode<PM>() != FOLD_FROM_SPEC) {
+                    if (in_half<PM>()) {
 #pragma unroll
                         for (int r = 0; r < H; ++r) {
                             const float2 t = ldc2(&a.ax.th[r * nk + k]);
@@ -617,10 +645,10 @@ struct Pass {
                         w[H] = cmul(s[H * rs + lk], ldc2(&a.ax.tc[(H - 1) * nk + k]));
                     }
                     Dft<r_, false>::run(w);
-                    if (in_half()) half_twiddle<r_, false>(w, std::make_integer_sequence<int, r_>{});
+                    if (in_half<PM>()) half_twiddle<r_, false>(w, std::make_integer_sequence<int, r_>{});
                 }
                 // spectral update; outputs q >= R/2 hold sg x (canonical bin)
-                if (mode() == FOLD_STEP) {
+                if (mode<PM>() == FOLD_STEP) {
                     const Slots sl = slots(p, k, nv == 2 * P());
                     if constexpr (!ahead_u) {
                         // all slots are read before any is written (bins of a
@@ -632,7 +660,7 @@ struct Pass {
                     } else {
                         update(w, uw, sl, k, kb);
                     }
-                } else if (mode() == FOLD_TO_SPEC) {
+                } else if (mode<PM>() == FOLD_TO_SPEC) {
                     const Slots sl = slots(p, k, false);
 #pragma unroll
                     for (int q = 0; q < r_; ++q) {
@@ -640,7 +668,7 @@ struct Pass {
                         const float sq = 2 * q < r_ ? 1.0f : sg;
                         store_slot(sl, k, kb, q, make_float2(rmul(sq, w[q].y), -rmul(sq, w[q].x)));
                     }
-                } else if (mode() == FOLD_FROM_SPEC) {
+                } else if (mode<PM>() == FOLD_FROM_SPEC) {
                     const Slots sl = slots(p, k, false);
                     const float sc = 1.0f / (float)L();
 #pragma unroll
@@ -653,13 +681,13 @@ struct Pass {
 #pragma unroll
                     for (int q = 0; q < r_; ++q) {
                         // the signs of the canonical bin's two uses cancel
-                        const float f = ldc(&a.f[bin(k, q)]);
-                        w[q] = mode() == FOLD_ORDER2 ? cscale(w[q], f)
+                        const float f = ldc(&(MODE == FOLD_CONV && PM == FOLD_GRAD_U ? a.f2 : a.f)[bin(k, q)]);
+                        w[q] = mode<PM>() == FOLD_ORDER2 ? cscale(w[q], f)
                                                      : make_float2(-rmul(f, w[q].y), rmul(f, w[q].x));
                     }
                 }
-                if (mode() == FOLD_TO_SPEC) return;
-                if (out_half()) {
+                if (mode<PM>() == FOLD_TO_SPEC) return;
+                if (out_half<PM>()) {
                     half_twiddle<r_, true>(w, std::make_integer_sequence<int, r_>{});
                     Dft<r_, true>::run(w);
 #pragma unroll
@@ -716,7 +744,7 @@ struct Pass {
         if (half) {
             mir = even ? 2 * e >= a_ : j >= n;
             i = mir ? 2 * n - 1 - j : j;
-            return true;
+            return !conv() || i < a.ax.cN;
         }
         mir = even ? 2 * e >= a_ : j > n;
         i = (mir ? 2 * n - j : j) - a.ax.lo;
@@ -728,15 +756,15 @@ struct Pass {
                 mir = false;
             }
         }
-        if (!even || e == 0 || 2 * e == a_) ok = ok && i >= 0 && i < a.ax.lp;
+        if (conv() || !even || e == 0 || 2 * e == a_) ok = ok && i >= 0 && i < a.ax.lp;
         return ok;
     }
     PSTD_HD void fetch_acc() {
         if constexpr (ahead && !onto_p) {
             by_full([&](auto full) {
-                const float* xa = base(MODE == FOLD_STEP ? a.acc_in : (const float*)a.out, nout());
+                const float* xa = base(MODE == FOLD_ORDER2 ? (const float*)a.out : a.acc_in, nout());
                 const float* xb = xa + line_step(nout());
-                const bool acc = MODE == FOLD_STEP || a.accumulate;
+                const bool acc = MODE != FOLD_ORDER2 || a.accumulate;
                 items((C::R / 2 + 1) * C::B, [&](int p, int w) {
                     const int r = w / C::B, t = w - r * C::B, j0 = C::R * t + r;
                     const bool la = full || va(p), lb = full || vb(p);
@@ -824,11 +852,79 @@ struct Pass {
             });
         });
     }
+    // Convolution pass, between its two derivatives: residue r, lane t of the
+    // half-nodes: the inverse's last radix, u += , and the first radix of the
+    // transform of the new u (the same positions).  The new u goes straight to
+    // memory (strided) or to the rows.
+    PSTD_HD void mid() {
+        with_radix<C::A>(A(), [&](auto RA) {
+            constexpr int a_ = decltype(RA)::value;
+            const float rsg = -a.ax.rho;
+            float* ua = base(a.u, nhalf());
+            float* ub = ua + line_step(nhalf());
+            items(R() / 2 * B(), [&](int p, int w) {
+                const int r = w / B(), t = w - r * B(), j0 = R() * t + r, dj = R() * B();
+                float2* s = at(r, p) + Ap() * t * ls();
+                const bool la = va(p), lb = vb(p);
+                const Off ps = pos_step(), lof = line_off(p, nhalf());
+                const Off od = lof + (Off)j0 * ps, om = lof + (Off)(2 * N() - 1 - j0) * ps, step = (Off)dj * ps;
+                float2 x[a_], u[a_];
+#pragma unroll
+                for (int e = 0; e < a_; ++e) {
+                    int i;
+                    bool mir;
+                    const bool ok = out_index<a_>(e, false, j0 + dj * e, true, i, mir);
+                    const Off off = mir ? om - (Off)e * step : od + (Off)e * step;
+                    u[e] = make_float2(ok && la ? ld(ua, off) : 0.0f, ok && lb ? ld(ub, off) : 0.0f);
+                }
+#pragma unroll
+                for (int k = 0; k < a_; ++k) {
+                    x[k] = s[k * ls()];
+                    if (k > 0) x[k] = cmulc(x[k], ldc2(&a.ax.tw[k * B() + t]));
+                }
+                Dft<a_, true>::run(x);
+#pragma unroll
+                for (int e = 0; e < a_; ++e) {
+                    int i;
+                    bool mir;
+                    const bool ok = out_index<a_>(e, false, j0 + dj * e, true, i, mir);
+                    const Off off = mir ? om - (Off)e * step : od + (Off)e * step;
+                    const float sgn = mir ? rsg : 1.0f;
+                    const float2 v = make_float2(rfma(sgn, x[e].x, u[e].x), rfma(sgn, x[e].y, u[e].y));
+                    if constexpr (STR) {
+                        if (ok && la) put(ua, off, v.x);
+                        if (ok && lb) put(ub, off, v.y);
+                    } else if (ok) {
+                        float* q = st + 2 * p * row_pitch(a.ax) + row_word(i);
+                        q[0] = v.x;
+                        q[row_pitch(a.ax)] = v.y;
+                    }
+                    x[e] = make_float2(ok && la ? rmul(sgn, v.x) : 0.0f, ok && lb ? rmul(sgn, v.y) : 0.0f);
+                }
+                Dft<a_, false>::run(x);
+#pragma unroll
+                for (int k = 0; k < a_; ++k) {
+                    if (k > 0) x[k] = cmul(x[k], ldc2(&a.ax.tw[k * B() + t]));
+                    s[k * ls()] = x[k];
+                }
+            });
+        });
+    }
+    // the new u of contiguous lines from their rows
+    PSTD_HD void finish_u() {
+        if constexpr (!STR) {
+            const int len = nhalf(), pitch = row_pitch(a.ax);
+            float* y = base(a.u, len);
+            const int wid = tid >> 5, lane = tid & 31, nw = (nthr + 31) >> 5;
+            for (int l = wid; l < nv; l += nw)
+                for (int i = lane; i < len; i += 32) y[l * (int64_t)len + i] = st[l * pitch + row_word(i)];
+        }
+    }
     // *y = its new value from contribution c
     PSTD_HD void emit(float* y, bool ok, float c) const {
         if (!ok) return;
         const int64_t off = y - a.out;
-        if (mode() == FOLD_STEP) {
+        if (mode() == FOLD_STEP || mode() == FOLD_CONV) {
             *y = radd(a.acc_in[off], c);
             return;
         }
@@ -864,7 +960,8 @@ struct Pass {
                 asm volatile("prefetch.global.L1 [%0];" ::"l"((const char*)p + i));
         };
         touch(a.ax.tw, M() * 8);
-        touch(in_half() || out_half() ? a.ax.th : a.ax.tc, R() / 2 * a.ax.nk * 8);
+        if (in_half() || out_half() || MODE == FOLD_CONV) touch(a.ax.th, R() / 2 * a.ax.nk * 8);
+        if (!in_half() || !out_half()) touch(a.ax.tc, R() / 2 * a.ax.nk * 8);
         if (a.coef) touch(a.coef, (N() + 1) * 8);
 #endif
     }
@@ -881,6 +978,32 @@ __device__ __forceinline__ void fold_pass(const FoldArgs& a, unsigned item, void
     // turn for this grid to end)
     pdl_wait();
     pdl_trigger();
+    if constexpr (MODE == FOLD_CONV) {
+        ps.template p1<FOLD_GRAD_P>();
+        __syncthreads();
+        ps.template p2<FOLD_GRAD_P>();
+        __syncthreads();
+        ps.template p3<FOLD_GRAD_P>();
+        __syncthreads();
+        ps.template p4<FOLD_GRAD_P>();
+        __syncthreads();
+        ps.mid();
+        __syncthreads();
+        ps.finish_u();
+        ps.template p2<FOLD_GRAD_U>();
+        __syncthreads();
+        ps.template p3<FOLD_GRAD_U>();
+        ps.fetch_acc();
+        __syncthreads();
+        ps.template p4<FOLD_GRAD_U>();
+        __syncthreads();
+        ps.p5();
+        if constexpr (!STR) {
+            __syncthreads();
+            ps.finish();
+        }
+        return;
+    }
     if constexpr (!STR) ps.fetch_u();
     ps.p1();
     if constexpr (STR) ps.fetch_u();

@@ -8,9 +8,19 @@ const void* fold_any_misc_c();
 #define DECL(U) const void* fold_unit_##U(int R, int A, int B, int P, bool strided, int mode);
 PSTD_FOLD_UNITS(DECL)
 #undef DECL
+#define DECL(U) const void* conv_unit_##U(int R, int A, int B, bool strided);
+PSTD_CONV_UNITS(DECL)
+#undef DECL
 
 const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) {
     fixed = true;
+    if (mode == FOLD_CONV) {
+#define TRY(U) \
+    if (const void* k = conv_unit_##U(x.R, x.A, x.B, strided)) return k;
+        PSTD_CONV_UNITS(TRY)
+#undef TRY
+        return nullptr;
+    }
     if (!x.wide && (mode == FOLD_STEP || mode == FOLD_ORDER2 || mode == FOLD_LINE)) {
 #define TRY(U) \
     if (const void* k = fold_unit_##U(x.R, x.A, x.B, x.P, strided, mode)) return k;
@@ -39,7 +49,7 @@ cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cu
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = a.mode == FOLD_STEP || a.mode == FOLD_ORDER2 ? 1 : 0;
+    cfg.numAttrs = a.mode == FOLD_STEP || a.mode == FOLD_ORDER2 || a.mode == FOLD_CONV ? 1 : 0;
     void* args[] = {(void*)&a};
     return cudaLaunchKernelExC(&cfg, k, args);
 }
@@ -56,7 +66,8 @@ cudaError_t fold_launch_line(const FoldArgs& a, int64_t nsteps, const FoldLaunch
 }
 
 cudaError_t fold_set_smem(const FoldAxis& x, bool strided, int bytes) {
-    for (int mode : {(int)FOLD_STEP, (int)FOLD_ORDER2, (int)FOLD_GRAD_P}) {
+    for (int mode : {(int)(x.cN ? FOLD_CONV : FOLD_STEP), (int)FOLD_ORDER2, (int)FOLD_GRAD_P}) {
+        if (x.cN && mode == FOLD_ORDER2) continue;
         bool fixed = false;
         const void* k = fold_kernel(x, strided, mode, fixed);
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -93,5 +93,15 @@
     X(8, 8, 12, 4, 4) \
     X(10, 9, 15, 4, 2) \
     X(12, 12, 12, 4, 2)
+// Embeddings of the convolution passes (lines of N cells with no schedule of
+// their own, 65 <= N <= 1280): the smallest length that is at least 4N, 4 to
+// 12 percent apart, as X(R, A, B); 2 line pairs per CTA on strided axes, 1 on
+// contiguous ones.
+#define PSTD_CONV_U0(X) X(8, 6, 6) X(6, 8, 9) X(8, 8, 10) X(10, 10, 10) X(10, 12, 12) X(8, 16, 16) X(12, 15, 16) X(18, 16, 16)
+#define PSTD_CONV_U1(X) X(8, 5, 8) X(6, 8, 10) X(8, 9, 10) X(8, 9, 15) X(10, 10, 16) X(10, 15, 15) X(12, 16, 16) X(20, 16, 16)
+#define PSTD_CONV_U2(X) X(8, 5, 9) X(8, 8, 8) X(8, 10, 10) X(10, 10, 12) X(12, 12, 12) X(10, 15, 16) X(16, 15, 15)
+#define PSTD_CONV_U3(X) X(8, 5, 10) X(8, 8, 9) X(10, 9, 10) X(8, 10, 16) X(10, 12, 16) X(10, 16, 16) X(16, 16, 16)
+#define PSTD_CONV_ALL(X) PSTD_CONV_U0(X) PSTD_CONV_U1(X) PSTD_CONV_U2(X) PSTD_CONV_U3(X)
+#define PSTD_CONV_UNITS(X) X(0) X(1) X(2) X(3)
 #define PSTD_FOLD_ALL(X) PSTD_FOLD_U0(X) PSTD_FOLD_U1(X) PSTD_FOLD_U2(X) PSTD_FOLD_U3(X) PSTD_FOLD_U4(X) PSTD_FOLD_U5(X) PSTD_FOLD_U6(X) PSTD_FOLD_U7(X) PSTD_FOLD_U8(X) PSTD_FOLD_U9(X)
 #define PSTD_FOLD_UNITS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9)

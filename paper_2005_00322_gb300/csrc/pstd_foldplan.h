@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cmath>
+#include <complex>
 #include <vector>
 
 #include "pstd_fold.cuh"
@@ -81,6 +82,24 @@ inline bool fold_choose(int L, FoldChoice& best) {
     return best.R > 0;
 }
 
+// Embedding of a line of N cells: the smallest compiled length L >= 4N.
+inline bool conv_choose(int N, FoldChoice& best) {
+    static const FoldChoice all[] = {
+#define ENTRY(R, A, B) {R, A, B, 2, 1},
+        PSTD_CONV_ALL(ENTRY)
+#undef ENTRY
+    };
+    int least = 0;
+    for (const FoldChoice& f : all) {
+        const int L = f.R * f.A * f.B;
+        if (L >= 4 * N && (least == 0 || L < least)) {
+            least = L;
+            best = f;
+        }
+    }
+    return least > 0;
+}
+
 struct FoldTables {
     std::vector<float2> tw, tc, th;
 };
@@ -117,6 +136,38 @@ inline void fold_axis(int N, int left, int right, const FoldChoice& ch, FoldAxis
             t.tc[(size_t)r * x.nk + k] = unit((long)(r + 1) * (2 * k + x.g), x.L);
             t.th[(size_t)r * x.nk + k] = unit((long)(2 * r + 1) * (2 * k + x.g), 2L * x.L);
         }
+}
+
+// The embedding of an axis of N cells (walls as above) on choice `ch`: a
+// folded axis of N' = L / 2 cells between two walls of the left wall's kind,
+// storing the line's own nodes and half-nodes only.
+inline void fold_axis_conv(int N, int left, int right, const FoldChoice& ch, FoldAxis& x, FoldTables& t) {
+    fold_axis(ch.R * ch.A * ch.B / 2, left, left, ch, x, t);
+    x.cN = N;
+    x.lp = (right ? N - 1 : N) - left + 1;
+}
+// The staggered derivative's kernel at lag t = m + 1/2 (unit spacing), the
+// derivative of the period-L interpolation kernel (Nyquist bin included once):
+// group I sin(pi t) cot(pi t / L) / L, group II sin(pi t) / sin(pi t / L) / L.
+inline double stagger_kernel(int N, int g, int m) {
+    const double L = 2.0 * N, a = M_PI * (m + 0.5) / L, sn = std::sin(a);
+    return -(m & 1 ? -1.0 : 1.0) * M_PI / (L * L) * (g ? std::cos(a) : 1.0) / (sn * sn);
+}
+// Multiplier per bin of an embedded derivative, C = i f X: the spectrum of the
+// kernel cut off at |t| < 2N, over L; `fft` is a forward FP64 DFT in place.
+template <class Fft>
+std::vector<double> conv_coef(const FoldAxis& x, int g, double dx, Fft&& fft) {
+    const int N = x.cN, L = x.L;
+    std::vector<std::complex<double>> h((size_t)L, 0.0);
+    for (int m = 0; m < 2 * N; ++m) {
+        const double v = stagger_kernel(N, g, m);
+        h[(size_t)m] += v;
+        h[(size_t)(L - 1 - m)] -= v;         // odd: lag -(m + 1/2)
+    }
+    fft(h);
+    std::vector<double> f((size_t)x.N + 1);
+    for (int b = 0; b <= x.N; ++b) f[b] = (h[(size_t)b] * std::polar(1.0, -M_PI * b / L)).imag() / (L * dx);
+    return f;
 }
 
 // Threads of a CTA: one per element group of the widest phase.

@@ -167,6 +167,8 @@ struct Axis {
     float* d_fgrad[OP_COUNT] = {};    // derivative multipliers per bin (GRAD_P, GRAD_U, INIT_P)
     float* d_f2fold = nullptr;        // second-order multiplier per bin, on first use
     bool fold() const { return wl > 0 && wv == kFold; }
+    bool cfold = false;               // convolution passes on folded transforms (fax; wl == 0)
+    float* d_fconv[2] = {nullptr, nullptr};   // step multipliers p -> u, u -> p
     // BF16 three-way split form on tcgen05: the two operators' BF16 slices
     // (D1: N x lp, D2: lp x N) and their TMA tensor maps
     uint16_t* d_tc16[2] = {nullptr, nullptr};
@@ -809,6 +811,43 @@ int build_fold(pstd_plan_s* P, int i, const pstd::FoldChoice& ch, int os) {
     return PSTD_OK;
 }
 
+// Convolution passes of axis i on folded transforms.
+int build_conv(pstd_plan_s* P, int i, const pstd::FoldChoice& ch) {
+    Axis& a = P->ax[i];
+    const pstd_desc& d = P->desc;
+    pstd::FoldTables t;
+    FoldAxis& x = a.fax;
+    pstd::fold_axis_conv(a.N, a.bcl == PSTD_DIRICHLET, a.bcr == PSTD_DIRICHLET, ch, x, t);
+    x.nlines = a.nlines;
+    x.inner = a.inner;
+    a.strided = a.inner > 1;
+    x.P = a.strided ? ch.PS : ch.PC;
+    x.lgP = x.P == 2 ? 1 : 0;
+    a.fgeo.grid = (unsigned)(a.strided ? (a.nlines / a.inner) * ((a.inner + 2 * x.P - 1) / (2 * x.P))
+                                       : (a.nlines + 2 * x.P - 1) / (2 * x.P));
+    a.fgeo.threads = pstd::fold_threads(x);
+    a.fgeo.smem = pstd::fold::smem_bytes(x, a.strided);
+    std::vector<float2> tab(t.tw);
+    tab.insert(tab.end(), t.tc.begin(), t.tc.end());
+    tab.insert(tab.end(), t.th.begin(), t.th.end());
+    int rc;
+    if ((rc = upload(tab, &a.d_ftab)) != PSTD_OK) return rc;
+    x.tw = a.d_ftab;
+    x.tc = x.tw + t.tw.size();
+    x.th = x.tc + t.tc.size();
+    const std::vector<double> f1 = pstd::conv_coef(x, a.group2, a.dx, host_fft);
+    const struct { float** d; double scale; } out[5] = {
+        {&a.d_fconv[0], -d.dt / d.rho0}, {&a.d_fconv[1], -d.dt * d.rho0 * d.c0 * d.c0},
+        {&a.d_fgrad[OP_GRAD_P], 1.0}, {&a.d_fgrad[OP_GRAD_U], 1.0}, {&a.d_fgrad[OP_INIT_P], d.dt / (2.0 * d.rho0)}};
+    for (const auto& o : out) {
+        std::vector<float> f(f1.size());
+        for (size_t b = 0; b < f.size(); ++b) f[b] = (float)(f1[b] * o.scale);
+        if ((rc = upload(f, o.d)) != PSTD_OK) return rc;
+    }
+    a.cfold = true;
+    return PSTD_OK;
+}
+
 // Dense operators of the split forms of axis i (pstd_plan_opts.form 1, 2, 3).
 int build_forms(pstd_plan_s* P, int i) {
     Axis& a = P->ax[i];
@@ -903,6 +942,29 @@ int build_forms(pstd_plan_s* P, int i) {
 }
 
 
+// Tables of the shared-memory convolution route (LineOp kind 2), built where
+// that program runs the axis: at plan time unless the folded passes do, and then
+// on the first cooperative batch run.
+int build_conv_tables(pstd_plan_s* P, int i) {
+    Axis& a = P->ax[i];
+    if (a.kind != 2 || a.d_f[0]) return PSTD_OK;
+    const pstd_desc& d = P->desc;
+    const double scales[OP_COUNT] = {1.0, 1.0, -d.dt / d.rho0, -d.dt * d.rho0 * d.c0 * d.c0,
+                                     d.dt / (2.0 * d.rho0)};
+    const std::vector<std::complex<double>> conv[2] = {conv_table(a, 0), conv_table(a, 1)};
+    for (int o = OP_COUNT - 1; o >= 0; --o) {       // d_f[0], the mark that they are built, last
+        std::vector<float2> H(a.M2);
+        for (int n = 0; n < a.M2; ++n) {
+            const std::complex<double> c = conv[a.op[o].dir][n] * scales[o];
+            H[n] = make_float2((float)c.real(), (float)c.imag());
+        }
+        const int rc = upload(H, &a.d_f[o]);
+        if (rc != PSTD_OK) return rc;
+        a.op[o].f = a.d_f[o];
+    }
+    return PSTD_OK;
+}
+
 int build_axis(pstd_plan_s* P, int i) {
     Axis& a = P->ax[i];
     const pstd_desc& d = P->desc;
@@ -969,11 +1031,6 @@ int build_axis(pstd_plan_s* P, int i) {
     const double scales[OP_COUNT] = {1.0, 1.0, -d.dt / d.rho0, -d.dt * d.rho0 * d.c0 * d.c0,
                                      d.dt / (2.0 * d.rho0)};
     const int dirs[OP_COUNT] = {0, 1, 0, 1, 0};
-    std::vector<std::complex<double>> conv[2];
-    if (a.kind == 2) {
-        conv[0] = conv_table(a, 0);
-        conv[1] = conv_table(a, 1);
-    }
     for (int o = 0; o < OP_COUNT; ++o) {
         const int dir = dirs[o];
         LineOp& op = a.op[o];
@@ -997,13 +1054,7 @@ int build_axis(pstd_plan_s* P, int i) {
         op.seqlen = FL;
         op.fold = a.group2 ? -1.0f : 1.0f;
         if (a.kind == 2) {
-            std::vector<float2> H(a.M2);
-            for (int n = 0; n < a.M2; ++n) {
-                const std::complex<double> c = conv[dir][n] * scales[o];
-                H[n] = make_float2((float)c.real(), (float)c.imag());
-            }
-            if ((rc = upload(H, &a.d_f[o])) != PSTD_OK) return rc;
-            op.f = a.d_f[o];
+            // tables by build_conv_tables
         } else if (a.kind == 0) {
             std::vector<float2> f(a.L);
             for (int n = 0; n < a.L; ++n) {
@@ -1049,6 +1100,15 @@ int build_axis(pstd_plan_s* P, int i) {
             return build_fold(P, i, ch, ov == kFold ? os : -1);
         }
     }
+
+    // lines with no schedule: the convolution on folded transforms, steps and
+    // first derivatives
+    if (a.kind == 2 && !a.periodic && !a.mid && P->opts.form == 0) {
+        pstd::FoldChoice ch{};
+        if (pstd::conv_choose(a.N, ch) && (int64_t)(a.N + 1) * a.inner < (int64_t)1 << 30) return build_conv(P, i, ch);
+    }
+
+    if (a.kind == 2 && (rc = build_conv_tables(P, i)) != PSTD_OK) return rc;
 
     // register-FFT passes where a schedule exists.  Measured on GB300 (512^2,
     // 256^3, 384^3): the latency schedules (8 or 12 elements per lane) beat
@@ -1219,6 +1279,8 @@ void free_plan_memory(pstd_plan_s* P) {
         cudaFree(a.d_ftab);
         cudaFree(a.d_fcoef);
         cudaFree(a.d_f2fold);
+        cudaFree(a.d_fconv[0]);
+        cudaFree(a.d_fconv[1]);
         for (float* f : a.d_fgrad) cudaFree(f);
         cudaFree(a.d_f2);
         cudaFree(a.d_dense2);
@@ -1375,8 +1437,10 @@ FoldArgs fold_step(pstd_plan_s* P, int a, float* p, float* const* u) {
     Axis& A = P->ax[a];
     FoldArgs f{};
     f.ax = A.fax;
-    f.mode = pstd::FOLD_STEP;
+    f.mode = A.cfold ? pstd::FOLD_CONV : pstd::FOLD_STEP;
     f.coef = A.d_fcoef;
+    f.f = A.d_fconv[0];
+    f.f2 = A.d_fconv[1];
     f.in = p;
     f.u = u[a];
     f.acc_in = (a == P->ndim - 1) ? p : P->d_S;
@@ -1468,7 +1532,7 @@ int launch_step(pstd_plan_s* P, float* p, float* const* u, int64_t* launches) {
             ++*launches;
             continue;
         }
-        if (A.fold()) {
+        if (A.fold() || A.cfold) {
             CK(pstd::fold_launch(fold_step(P, a, p, u), A.strided, A.fgeo, P->stream));
             ++*launches;
             continue;
@@ -1496,7 +1560,7 @@ int launch_step(pstd_plan_s* P, float* p, float* const* u, int64_t* launches) {
 
 int launch_grad(pstd_plan_s* P, int axis, int opi, const float* in, float* out, int acc) {
     Axis& A = P->ax[axis];
-    if (A.fold()) {
+    if (A.fold() || A.cfold) {
         FoldArgs f{};
         f.ax = A.fax;
         f.mode = A.op[opi].dir == 0 ? pstd::FOLD_GRAD_P : pstd::FOLD_GRAD_U;
@@ -1745,6 +1809,12 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
                                     cudaStream_t st) {
     const int kind = pstd_internal_batch_persist_kind(plans, n);
     if (kind == 0) return PSTD_EUNSUPPORTED;
+    if (kind == 2)
+        for (int m = 0; m < n; ++m)
+            for (int a = 0; a < plans[m]->ndim; ++a) {
+                const int rc = build_conv_tables(plans[m], a);
+                if (rc != PSTD_OK) return rc;
+            }
     if (!*state) {
         *state = new (std::nothrow) pstd_batch_persist_s();
         if (!*state) return PSTD_ENOMEM;
@@ -1997,11 +2067,11 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
             if (e != cudaSuccess) rc = cuda_fail(e, "cudaFuncSetAttribute(split-precision pass)");
         }
         for (int i = 0; i < P->ndim && rc == PSTD_OK; ++i) {
-            if (!P->ax[i].wl) continue;
+            if (!P->ax[i].wl && !P->ax[i].cfold) continue;
             int dev = 0, optin = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-            e = P->ax[i].fold() ? pstd::fold_set_smem(P->ax[i].fax, P->ax[i].strided, optin)
+            e = P->ax[i].fold() || P->ax[i].cfold ? pstd::fold_set_smem(P->ax[i].fax, P->ax[i].strided, optin)
                                 : wsmem(P->ax[i].L, P->ax[i].wv, optin);
             if (e != cudaSuccess) rc = cuda_fail(e, "cudaFuncSetAttribute(register-FFT pass)");
         }
