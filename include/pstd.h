@@ -492,6 +492,18 @@ int pstd_nn_gemm(const pstd_gemm_desc* d, void* stream);
  * tile is then left unwritten.  Errors: PSTD_EINVAL, PSTD_ECUDA. */
 int pstd_nn_gemm_tf32(const pstd_gemm_desc* d, int* status, void* stream);
 
+/* One spectral layer's output in one pass over the field, out and v being
+ * [B][C][X][Y] (out must not alias v):
+ *   z = sum_i W[o][i] v[b][i][x][y] + sum_k A[b][o][x][k] T[k][y] + bias[o]
+ *   out = act(z) (act 0 = identity, 1 = relu), or 0 where mask is given and
+ *   mask[b][o][x][y] > 0 does not hold (the adjoint of a relu).
+ * w_transposed: W is stored [i][o]; t_by_mode: T is stored [k][y], else [y][k];
+ * bias and mask may be NULL.  C <= 32 and K <= 32, B <= 65535.  Errors:
+ * PSTD_EINVAL, PSTD_EUNSUPPORTED (larger C, K, B), PSTD_ECUDA. */
+int pstd_nn_mix(const float* W, int w_transposed, const float* v, const float* A, const float* T, int t_by_mode,
+                const float* bias, const float* mask, float* out, int64_t B, int C, int X, int Y, int K, int act,
+                void* stream);
+
 /* Tensors below are [B][C][P] (B samples, C channels, P points) or [B][P];
  * bias_act, lift and proj_bwd need B C <= 65535, proj B <= 65535.
  * y = act(x + bias[c]) with act 0 = identity, 1 = relu; bias may be NULL. */

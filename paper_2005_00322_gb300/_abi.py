@@ -59,6 +59,8 @@ SIGNATURES = {
     "pstd_nn_gemm_tf32": (c_int, [c_void_p, c_void_p, c_void_p]),
     "pstd_nn_bias_act": (c_int, [c_void_p, c_void_p, c_void_p, c_int64, c_int, c_int64, c_int, c_void_p]),
     "pstd_nn_act_bwd": (c_int, [c_void_p, c_void_p, c_void_p, c_int64, c_int, c_void_p]),
+    "pstd_nn_mix": (c_int, [c_void_p, c_int, c_void_p, c_void_p, c_void_p, c_int, c_void_p, c_void_p, c_void_p,
+                            c_int64, c_int, c_int, c_int, c_int, c_int, c_void_p]),
     "pstd_nn_lift": (c_int, [c_void_p, c_void_p, c_void_p, c_void_p, c_int64, c_int, c_int64, c_void_p]),
     "pstd_nn_proj": (c_int, [c_void_p, c_void_p, c_void_p, c_void_p, c_int64, c_int, c_int64, c_void_p]),
     "pstd_nn_proj_bwd": (c_int, [c_void_p, c_void_p, c_void_p, c_int64, c_int, c_int64, c_void_p]),

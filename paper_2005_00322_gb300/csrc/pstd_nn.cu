@@ -25,7 +25,8 @@ namespace {
 // thread) over 16-wide k slices staged in shared memory.  Tile shapes:
 // 64 x 64 for square-ish products, 256 x 16 / 16 x 256 for the tall or wide
 // products with a mode count (16) on one side, 16 x 16 for the small per-line
-// transforms.
+// transforms, 32 x 32 for the channel-by-channel products (the weight gradients
+// of 32 channels over 2048 chunks of 256 points: 152 us on 16 x 16 tiles).
 template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__(256) k_sgemm(pstd_gemm_desc d) {
     static_assert((BM / TM) * (BN / TN) == 256, "256 threads");
@@ -129,13 +130,17 @@ __global__ void k_act_bwd(const float* dy, const float* pre, float* dx, int64_t 
         dx[t] = (act == 1 && pre[t] <= 0.0f) ? 0.0f : dy[t];
 }
 
-// v[b, c, i] = w[c] p[b, i] + bias[c]
+// v[b, c, i] = w[c] p[b, i] + bias[c]  (blockIdx.y = b).  A thread writes all
+// channels of its points: with a row of CTAs per (b, c) and one point per
+// thread, 256 x 32 rows of 16383 points took 536 us for 537 MB.
 __global__ void k_lift(const float* p, const float* w, const float* bias, float* v, int C, int64_t P) {
-    const int64_t r = blockIdx.y, b = r / C;
-    const int c = (int)(r - b * C);
-    const float wc = w[c], bc = bias[c];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x)
-        v[r * P + i] = fmaf(wc, p[b * P + i], bc);
+    const int64_t b = blockIdx.y;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
+        const float x = p[b * P + i];
+        float* q = v + b * C * P + i;
+#pragma unroll 8
+        for (int c = 0; c < C; ++c, q += P) *q = fmaf(w[c], x, bias[c]);
+    }
 }
 
 // out[b, i] = sum_c w[c] v[b, c, i] + bias  (blockIdx.y = b)
@@ -148,40 +153,105 @@ __global__ void k_proj(const float* v, const float* w, const float* bias, float*
     }
 }
 
-// dv[b, c, i] = w[c] dout[b, i]
+// dv[b, c, i] = w[c] dout[b, i]  (blockIdx.y = b; as k_lift)
 __global__ void k_proj_bwd(const float* dout, const float* w, float* dv, int C, int64_t P) {
-    const int64_t r = blockIdx.y, b = r / C;
-    const float wc = w[r - b * C];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x)
-        dv[r * P + i] = wc * dout[b * P + i];
+    const int64_t b = blockIdx.y;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
+        const float x = dout[b * P + i];
+        float* q = dv + b * C * P + i;
+#pragma unroll 8
+        for (int c = 0; c < C; ++c, q += P) *q = w[c] * x;
+    }
 }
 
-// g[c] = sum_{b, i} x[b, c, i] * (y ? y[b, c or -, i] : 1); y indexed [b, i] when ybc == 0
-__global__ void k_chan_dot(const float* x, const float* y, int ybc, float* g, int64_t B, int C, int64_t P) {
-    const int c = blockIdx.x;
-    double acc = 0.0;
-    for (int64_t b = 0; b < B; ++b) {
-        const float* xr = x + (b * C + c) * P;
-        const float* yr = y ? (ybc ? y + (b * C + c) * P : y + b * P) : nullptr;
-        for (int64_t i = threadIdx.x; i < P; i += blockDim.x)
-            acc += (double)xr[i] * (yr ? (double)yr[i] : 1.0);
-    }
+// Sums in FP64 run at a few operations per clock and SM, so a reduction is
+// spread over the GPU: kRed CTAs of one cluster each add up a share, and the
+// first adds the shares through distributed shared memory in a fixed order
+// (no workspace, no atomics, the same bits each time).
+constexpr int kRed = 8;
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// Sum over the cluster's CTAs of `acc` over their threads (256), valid in
+// thread 0 of rank 0.
+__device__ double cluster_sum(double acc) {
     __shared__ double red[256];
+    __shared__ double part;
     red[threadIdx.x] = acc;
     __syncthreads();
     for (int s = blockDim.x / 2; s > 0; s >>= 1) {
         if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) g[c] = (float)red[0];
+    if (threadIdx.x == 0) part = red[0];
+    cluster_sync();
+    double tot = 0.0;
+    if (cluster_rank() == 0 && threadIdx.x == 0) {
+        const unsigned mine = (unsigned)__cvta_generic_to_shared(&part);
+        for (unsigned r = 0; r < kRed; ++r) {
+            unsigned at;
+            double v;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine), "r"(r));
+            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(at));
+            tot += v;
+        }
+    }
+    cluster_sync();          // no CTA leaves while its share may be read
+    return tot;
 }
 
-// out[j] = sum_b x[b, j]   (sum over the leading dimension)
-__global__ void k_sum_lead(const float* x, float* out, int64_t B, int64_t n) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+// g[c] = sum_{b, i} x[b, c, i] * (y ? y[b, c or -, i] : 1); y indexed [b, i] when ybc == 0
+// One cluster of kRed CTAs per channel.  With one CTA per channel (32 of the
+// SMs) 32 channels of 32 x 16383 points took 138 us of FP64 adds alone.
+__global__ void __launch_bounds__(256) k_chan_dot(const float* x, const float* y, int ybc, float* g, int64_t B, int C,
+                                                  int64_t P) {
+    const int c = blockIdx.x / kRed;
+    // four independent chains of adds and loads per thread
+    double acc[4] = {};
+    constexpr int64_t step = (int64_t)kRed * 256;
+    for (int64_t b = 0; b < B; ++b) {
+        const float* xr = x + (b * C + c) * P;
+        const float* yr = y ? (ybc ? y + (b * C + c) * P : y + b * P) : nullptr;
+        int64_t i = (int64_t)cluster_rank() * 256 + threadIdx.x;
+        for (; i + 3 * step < P; i += 4 * step) {
+            float xv[4], yv[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                xv[q] = xr[i + q * step];
+                yv[q] = yr ? yr[i + q * step] : 1.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[q] += (double)xv[q] * (double)yv[q];
+        }
+        for (; i < P; i += step) acc[0] += (double)xr[i] * (yr ? (double)yr[i] : 1.0);
+    }
+    const double tot = cluster_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+    if (cluster_rank() == 0 && threadIdx.x == 0) g[c] = (float)tot;
+}
+
+// out[j] = sum_b x[b, j] (sum over the leading dimension): a CTA takes 8
+// columns, its 32 groups of 8 threads every 32nd row each.
+__global__ void __launch_bounds__(256) k_sum_lead(const float* x, float* out, int64_t B, int64_t n) {
+    const int col = threadIdx.x & 7, grp = threadIdx.x >> 3;
+    __shared__ double red[32][8];
+    for (int64_t j0 = (int64_t)blockIdx.x * 8; j0 < n; j0 += (int64_t)gridDim.x * 8) {
+        const int64_t j = j0 + col;
         double acc = 0.0;
-        for (int64_t b = 0; b < B; ++b) acc += x[b * n + j];
-        out[j] = (float)acc;
+        if (j < n)
+            for (int64_t b = grp; b < B; b += 32) acc += x[b * n + j];
+        red[grp][col] = acc;
+        __syncthreads();
+        if (grp == 0 && j < n) {
+            double t = 0.0;
+            for (int q = 0; q < 32; ++q) t += red[q][col];
+            out[j] = (float)t;
+        }
+        __syncthreads();
     }
 }
 
@@ -212,18 +282,19 @@ __device__ double block_sum(double v) {
     return r;
 }
 
-// Mean squared error of out against target (one CTA): loss[0] = mean (out - t)^2,
-// dout = (2 / n) (out - t).
-__global__ void k_mse(const float* out, const float* target, float* dout, float* loss, int64_t n) {
+// Mean squared error of out against target (one cluster): loss[0] =
+// mean (out - t)^2, dout = (2 / n) (out - target).
+__global__ void __launch_bounds__(256) k_mse(const float* out, const float* target, float* dout, float* loss,
+                                             int64_t n) {
     double acc = 0.0;
     const float s = 2.0f / (float)n;
-    for (int64_t t = threadIdx.x; t < n; t += blockDim.x) {
+    for (int64_t t = cluster_rank() * blockDim.x + threadIdx.x; t < n; t += kRed * blockDim.x) {
         const float df = out[t] - target[t];
         acc += (double)df * (double)df;
         if (dout) dout[t] = s * df;
     }
-    const double tot = block_sum(acc);
-    if (threadIdx.x == 0) loss[0] = (float)(tot / (double)n);
+    const double tot = cluster_sum(acc);
+    if (cluster_rank() == 0 && threadIdx.x == 0) loss[0] = (float)(tot / (double)n);
 }
 
 // Per sample b (one CTA each): err[b] = ||a_b - r_b||_2 / ||r_b||_2.
@@ -263,6 +334,146 @@ __global__ void k_row_scale(const float* x, const float* sc, float* y, int64_t P
         y[b * P + i] = x[b * P + i] * f;
 }
 
+// ---- pointwise and spectral half of a layer in one pass ----------------------
+// out[b, o, x, y] = act( sum_i W[o, i] v[b, i, x, y] + sum_k A[b, o, x, k] T[k, y] + bias[o] ),
+// or, with `mask`, that value where mask > 0 and 0 elsewhere.  As separate
+// products, bias and activation the field went through memory seven times;
+// here v is read and out written once.  Each sum runs in index order and they
+// are added last, so every value has the bits of the separate products (a relu
+// argument near zero keeps its sign).
+// A CTA of 4 warps takes kMixX consecutive x of a sample and 128 y, the next
+// x's rows arriving (cp.async, second buffer) behind the current one's
+// products: lanes walk y (4 each, 32 apart, so shared reads and global accesses
+// are full lines), each warp has 8 output channels (12 shared reads feed 64
+// multiply-adds).
+constexpr int kMixC = 32, kMixK = 32, kMixX = 8, kMixY = 128;
+struct MixArgs {
+    const float* W;
+    int64_t sWo, sWi;
+    const float* v;
+    const float* A;
+    const float* T;
+    int64_t sTk, sTy;
+    const float* bias;
+    const float* mask;
+    float* out;
+    int C, X, Y, K, act;
+};
+__device__ __forceinline__ void copy4(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+// acc[m][q] += sum_j cf[j][m] rows[j][q], j ascending
+__device__ __forceinline__ void mix_rows(float (&acc)[8][4], const float* cf, const float* rows, int n) {
+    const float4* cp = (const float4*)cf;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j, rows += kMixY, cp += kMixC / 4) {
+        const float4 c0 = cp[0], c1 = cp[1];
+        const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+        float r[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) r[q] = rows[32 * q];
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][q] = fmaf(c[m], r[q], acc[m][q]);
+    }
+}
+inline size_t mix_smem(int C, int K) {
+    return (size_t)(2 * C * kMixY + K * kMixY + C * kMixC + 2 * K * kMixC) * sizeof(float);
+}
+__global__ void __launch_bounds__(128) k_mix(MixArgs a) {
+    extern __shared__ float sm[];
+    float* const vr = sm;                               // [2][C][128]
+    float* const tr = vr + 2 * a.C * kMixY;             // [K][128]
+    float* const wc = tr + a.K * kMixY;                 // [C][32]: W of (input, output channel)
+    float* const ac = wc + a.C * kMixC;                 // [2][K][32]: A of (mode, output channel)
+    const int tid = threadIdx.x, lane = tid & 31, wrp = tid >> 5;
+    const int y0 = blockIdx.x * kMixY, x0 = blockIdx.y * kMixX;
+    const int ny = a.Y - y0 < kMixY ? a.Y - y0 : kMixY;
+    const int64_t b = blockIdx.z, P = (int64_t)a.X * a.Y;
+    const int x1 = x0 + kMixX < a.X ? x0 + kMixX : a.X;
+    auto issue = [&](int x, int buf) {
+        float* d = vr + buf * a.C * kMixY;
+        for (int i = wrp; i < a.C; i += 4) {
+            const float* src = a.v + (b * a.C + i) * P + (int64_t)x * a.Y + y0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int y = lane + 32 * q;
+                if (y < ny) copy4(&d[i * kMixY + y], &src[y]);
+            }
+        }
+        float* e = ac + buf * a.K * kMixC;
+        for (int t = tid; t < a.K * a.C; t += 128) {
+            const int o = t / a.K, k = t - o * a.K;
+            copy4(&e[k * kMixC + o], &a.A[((b * a.C + o) * a.X + x) * a.K + k]);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    issue(x0, 0);
+    // columns and channels past the end stay zero in both buffers
+    for (int t = tid; t < 2 * a.C * kMixY; t += 128)
+        if (t % kMixY >= ny) vr[t] = 0.0f;
+    for (int t = tid; t < 2 * a.K * kMixC; t += 128)
+        if (t % kMixC >= a.C) ac[t] = 0.0f;
+    for (int t = tid; t < a.C * kMixC; t += 128) {
+        const int i = t / kMixC, o = t % kMixC;
+        wc[t] = o < a.C ? a.W[o * a.sWo + i * a.sWi] : 0.0f;
+    }
+    for (int t = tid; t < a.K * kMixY; t += 128) {
+        const int k = t / kMixY, y = t % kMixY;
+        tr[t] = y < ny ? a.T[k * a.sTk + (y0 + y) * a.sTy] : 0.0f;
+    }
+    for (int x = x0; x < x1; ++x) {
+        const int buf = (x - x0) & 1;
+        if (x + 1 < x1) {
+            issue(x + 1, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        float aw[8][4] = {}, as[8][4] = {};
+        mix_rows(as, ac + buf * a.K * kMixC + wrp * 8, tr + lane, a.K);
+        mix_rows(aw, wc + wrp * 8, vr + buf * a.C * kMixY + lane, a.C);
+        __syncthreads();                       // this buffer may be refilled
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const int o = wrp * 8 + m;
+            if (o >= a.C) break;
+            const int64_t off = (b * a.C + o) * P + (int64_t)x * a.Y + y0;
+            const float bv = a.bias ? a.bias[o] : 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int y = lane + 32 * q;
+                if (y >= ny) continue;
+                float z = aw[m][q] + as[m][q];
+                if (a.bias) z += bv;
+                if (a.act == 1) z = fmaxf(z, 0.0f);
+                if (a.mask && a.mask[off + y] <= 0.0f) z = 0.0f;
+                a.out[off + y] = z;
+            }
+        }
+    }
+}
+
+// Launch on clusters of kRed CTAs.
+template <class... KA, class... CA>
+cudaError_t launch_cluster(void (*k)(KA...), unsigned grid, cudaStream_t st, CA... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kRed;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<KA>(args)...);
+}
+
 dim3 row_grid(int64_t rows, int64_t P) {
     int64_t bx = (P + 255) / 256;
     return dim3((unsigned)(bx < 64 ? (bx > 0 ? bx : 1) : 64), (unsigned)rows);
@@ -287,10 +498,10 @@ int pstd_nn_gemm(const pstd_gemm_desc* d, void* stream) {
     if (nb2 > 1 && (d->K_last < 0 || d->K_last > d->K || (d->K_last > 0 && (!d->A || !d->B)))) return PSTD_EINVAL;
     if (d->batch * nb2 > 65535 || (d->M + 255) / 256 > 65535) return PSTD_EINVAL;
     // the tile shape that computes the fewest padded outputs (ties: 64 x 64)
-    static const int shapes[4][2] = {{64, 64}, {256, 16}, {16, 256}, {16, 16}};
+    static const int shapes[5][2] = {{64, 64}, {256, 16}, {16, 256}, {16, 16}, {32, 32}};
     int best = 0;
     int64_t best_cost = -1;
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < 5; ++t) {
         const int64_t bm = shapes[t][0], bn = shapes[t][1];
         const int64_t gm = (d->M + bm - 1) / bm;
         if (gm > 65535) continue;
@@ -306,8 +517,44 @@ int pstd_nn_gemm(const pstd_gemm_desc* d, void* stream) {
         case 0: k_sgemm<64, 64, 4, 4><<<grid, 256, 0, st>>>(*d); break;
         case 1: k_sgemm<256, 16, 4, 4><<<grid, 256, 0, st>>>(*d); break;
         case 2: k_sgemm<16, 256, 4, 4><<<grid, 256, 0, st>>>(*d); break;
+        case 4: k_sgemm<32, 32, 2, 2><<<grid, 256, 0, st>>>(*d); break;
         default: k_sgemm<16, 16, 1, 1><<<grid, 256, 0, st>>>(*d); break;
     }
+    return cuda_rc(cudaGetLastError());
+}
+
+int pstd_nn_mix(const float* W, int w_transposed, const float* v, const float* A, const float* T, int t_by_mode,
+                const float* bias, const float* mask, float* out, int64_t B, int C, int X, int Y, int K, int act,
+                void* stream) {
+    if (!W || !v || !A || !T || !out || B < 0 || C < 1 || X < 0 || Y < 0 || K < 1 || (act != 0 && act != 1))
+        return PSTD_EINVAL;
+    if (C > kMixC || K > kMixK || B > 65535 || (X + kMixX - 1) / kMixX > 65535) return PSTD_EUNSUPPORTED;
+    if (B == 0 || X == 0 || Y == 0) return PSTD_OK;
+    MixArgs a;
+    a.W = W;
+    a.sWo = w_transposed ? 1 : C;
+    a.sWi = w_transposed ? C : 1;
+    a.v = v;
+    a.A = A;
+    a.T = T;
+    a.sTk = t_by_mode ? Y : 1;
+    a.sTy = t_by_mode ? 1 : K;
+    a.bias = bias;
+    a.mask = mask;
+    a.out = out;
+    a.C = C;
+    a.X = X;
+    a.Y = Y;
+    a.K = K;
+    a.act = act;
+    const dim3 grid((unsigned)((Y + kMixY - 1) / kMixY), (unsigned)((X + kMixX - 1) / kMixX), (unsigned)B);
+    const size_t smem = mix_smem(C, K);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_mix, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)mix_smem(kMixC, kMixK));
+        if (e != cudaSuccess) return PSTD_ECUDA;
+    }
+    k_mix<<<grid, 128, smem, (cudaStream_t)stream>>>(a);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -329,7 +576,7 @@ int pstd_nn_lift(const float* p, const float* w, const float* bias, float* v, in
                  void* stream) {
     if (!p || !w || !bias || !v || C < 1 || B < 0 || P < 0 || B * C > 65535) return PSTD_EINVAL;
     if (B == 0 || P == 0) return PSTD_OK;
-    k_lift<<<row_grid(B * C, P), 256, 0, (cudaStream_t)stream>>>(p, w, bias, v, C, P);
+    k_lift<<<row_grid(B, P), 256, 0, (cudaStream_t)stream>>>(p, w, bias, v, C, P);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -344,20 +591,21 @@ int pstd_nn_proj(const float* v, const float* w, const float* bias, float* out, 
 int pstd_nn_proj_bwd(const float* dout, const float* w, float* dv, int64_t B, int C, int64_t P, void* stream) {
     if (!dout || !w || !dv || C < 1 || B < 0 || P < 0 || B * C > 65535) return PSTD_EINVAL;
     if (B == 0 || P == 0) return PSTD_OK;
-    k_proj_bwd<<<row_grid(B * C, P), 256, 0, (cudaStream_t)stream>>>(dout, w, dv, C, P);
+    k_proj_bwd<<<row_grid(B, P), 256, 0, (cudaStream_t)stream>>>(dout, w, dv, C, P);
     return cuda_rc(cudaGetLastError());
 }
 
 int pstd_nn_chan_dot(const float* x, const float* y, int y_has_channels, float* g, int64_t B, int C, int64_t P,
                      void* stream) {
     if (!x || !g || C < 1 || B < 0 || P < 0 || C > 0x7fffffff) return PSTD_EINVAL;
-    k_chan_dot<<<C, 256, 0, (cudaStream_t)stream>>>(x, y, y_has_channels, g, B, C, P);
-    return cuda_rc(cudaGetLastError());
+    if (C > 0x7fffffff / kRed) return PSTD_EINVAL;
+    return cuda_rc(launch_cluster(k_chan_dot, (unsigned)C * kRed, (cudaStream_t)stream, x, y, y_has_channels, g, B, C, P));
 }
 
 int pstd_nn_sum_lead(const float* x, float* out, int64_t B, int64_t n, void* stream) {
     if (!x || !out || B < 1 || n < 0) return PSTD_EINVAL;
-    k_sum_lead<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(x, out, B, n);
+    if (n == 0) return PSTD_OK;
+    k_sum_lead<<<blocks_for(n * 32), 256, 0, (cudaStream_t)stream>>>(x, out, B, n);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -371,8 +619,7 @@ int pstd_nn_adam(float* w, const float* g, float* m, float* v, int64_t n, float 
 
 int pstd_nn_mse(const float* out, const float* target, float* dout, float* loss, int64_t n, void* stream) {
     if (!out || !target || !loss || n < 1) return PSTD_EINVAL;
-    k_mse<<<1, 1024, 0, (cudaStream_t)stream>>>(out, target, dout, loss, n);
-    return cuda_rc(cudaGetLastError());
+    return cuda_rc(launch_cluster(k_mse, kRed, (cudaStream_t)stream, out, target, dout, loss, n));
 }
 
 int pstd_nn_rel_err(const float* a, const float* ref, float* err, int64_t B, int64_t P, void* stream) {

@@ -147,6 +147,16 @@ class SpectralOperator:
         self._status.zero_()
         return v
 
+    def _one_pass(self) -> bool:
+        """Whether a layer's pointwise mixing, last inverse transform, bias and
+        activation run as one kernel (pstd_nn_mix: FP32, up to 32 channels and modes)."""
+        return not self.tf32 and self.C <= 32 and self.K <= 32
+
+    def _mix(self, W, w_t, v, A, T, t_by_mode, bias, mask, out, act):
+        self._ck(self.lib.pstd_nn_mix(_ptr(W), int(w_t), _ptr(v), _ptr(A), _ptr(T), int(t_by_mode), _ptr(bias),
+                                      _ptr(mask), _ptr(out), v.shape[0], self.C, self.X, self.Y, self.K, act,
+                                      self._s()), "pstd_nn_mix")
+
     def _empty(self, *shape):
         return torch.empty(shape, dtype=torch.float32, device=self.device)
 
@@ -184,11 +194,14 @@ class SpectralOperator:
             # inverse transforms: A2[bc] = Ix U[bc], pre = A2 Iy^T
             self._gemm(B * C, X, K, K, self.Ix, (0, K, 1), U, (KK, K, 1), A2, (X * K, K, 1))
             vn = self._empty(B, C, X, Y)
-            self._gemm(1, B * C * X, Y, K, A2, (0, K, 1), self.Iy, (0, 1, K), vn, (0, Y, 1))
-            # pointwise channel mixing, bias, activation
-            self._gemm(B, C, P, C, W, (0, C, 1), v, (C * P, P, 1), vn, (C * P, P, 1), beta=1.0)
             act = 1 if l < self.L - 1 else 0
-            self._ck(self.lib.pstd_nn_bias_act(_ptr(vn), _ptr(b), _ptr(vn), B, C, P, act, s), "pstd_nn_bias_act")
+            if self._one_pass():
+                self._mix(W, False, v, A2, self.Iy, False, b, None, vn, act)
+            else:
+                self._gemm(1, B * C * X, Y, K, A2, (0, K, 1), self.Iy, (0, 1, K), vn, (0, Y, 1))
+                # pointwise channel mixing, bias, activation
+                self._gemm(B, C, P, C, W, (0, C, 1), v, (C * P, P, 1), vn, (C * P, P, 1), beta=1.0)
+                self._ck(self.lib.pstd_nn_bias_act(_ptr(vn), _ptr(b), _ptr(vn), B, C, P, act, s), "pstd_nn_bias_act")
             if keep:
                 cache["V"].append(Vh)
                 cache["v"].append(vn)
@@ -220,7 +233,7 @@ class SpectralOperator:
         for l in reversed(range(self.L)):
             vin, vout, Vh = cache["v"][l], cache["v"][l + 1], cache["V"][l]
             R, W = prm[f"R{l}"], prm[f"W{l}"]
-            if l < self.L - 1:      # relu: pre > 0 exactly where its output is > 0
+            if l < self.L - 1 and not self._one_pass():      # relu: pre > 0 exactly where its output is > 0
                 self._ck(self.lib.pstd_nn_act_bwd(_ptr(dv), _ptr(vout), _ptr(dv), dv.numel(), 1, s), "act_bwd")
             dpre = dv
             self._ck(self.lib.pstd_nn_chan_dot(_ptr(dpre), None, 0, _ptr(g[f"b{l}"]), B, C, P, s), "chan_dot")
@@ -230,7 +243,8 @@ class SpectralOperator:
                        split=(S, Lc, Lc, B * C * C, P - (S - 1) * Lc))
             self._ck(self.lib.pstd_nn_sum_lead(_ptr(Wp), _ptr(g[f"W{l}"]), S * B, C * C, s), "sum_lead")
             dvin = self._empty(B, C, X, Y)
-            self._gemm(B, C, P, C, W, (0, 1, C), dpre, (C * P, P, 1), dvin, (C * P, P, 1))
+            if not self._one_pass():
+                self._gemm(B, C, P, C, W, (0, 1, C), dpre, (C * P, P, 1), dvin, (C * P, P, 1))
             # adjoint of the inverse transforms: dU[bc] = Ix^T dpre[bc] Iy
             self._gemm(1, B * C * X, K, Y, dpre, (0, Y, 1), self.Iy, (0, K, 1), dA, (0, K, 1))
             self._gemm(B * C, K, K, X, self.Ix, (0, 1, K), dA, (X * K, K, 1), dU, (KK, K, 1))
@@ -239,7 +253,12 @@ class SpectralOperator:
             self._gemm(KK, C, B, C, R, (C * C, 1, C), dU, (1, KK, C * KK), dV, (1, KK, C * KK))
             # adjoint of the forward transforms: dvin += Tx^T dV[bc] Ty
             self._gemm(B * C, X, K, K, self.Tx, (0, 1, X), dV, (KK, K, 1), dA, (X * K, K, 1))
-            self._gemm(1, B * C * X, Y, K, dA, (0, K, 1), self.Ty, (0, Y, 1), dvin, (0, Y, 1), beta=1.0)
+            if self._one_pass():
+                # W^T dpre + dA Ty, through the previous layer's relu (its output
+                # vin is > 0 exactly where its argument is)
+                self._mix(W, True, dpre, dA, self.Ty, True, None, vin if l > 0 else None, dvin, 0)
+            else:
+                self._gemm(1, B * C * X, Y, K, dA, (0, K, 1), self.Ty, (0, Y, 1), dvin, (0, Y, 1), beta=1.0)
             dv = dvin
         self._ck(self.lib.pstd_nn_chan_dot(_ptr(dv), _ptr(p0), 0, _ptr(g["w_lift"]), B, C, P, s), "chan_dot")
         self._ck(self.lib.pstd_nn_chan_dot(_ptr(dv), None, 0, _ptr(g["b_lift"]), B, C, P, s), "chan_dot")
