@@ -161,7 +161,7 @@ int pstd_batch_plan(const pstd_desc* descs, int n, void* stream, pstd_batch_t** 
         if (e != cudaSuccess) { rc = pstd_internal_cuda_fail(e, "cudaEventCreate"); break; }
         B->joins.push_back(j);
         pstd_plan_t* P = nullptr;
-        rc = pstd_plan(&descs[m], s, &P);
+        rc = pstd_internal_plan_member(&descs[m], s, n, &P);
         if (rc == PSTD_OK) B->plans.push_back(P);
     }
     if (rc != PSTD_OK) {

@@ -108,17 +108,18 @@ const void* fold_fixed(int P, bool strided, int mode) {
         return nullptr;                                                                \
     }
 
-// Convolution pass on an embedding's radices (2 pairs per CTA strided, 1
+// Convolution pass on an embedding's radices (2 or 4 pairs per CTA strided, 1
 // contiguous), or null.
 template <int R, int A, int B>
-const void* conv_fixed(bool strided) {
-    return strided ? (const void*)fold::k_fold<fold::Cfg<R, A, B, 2>, true, FOLD_CONV>
-                   : (const void*)fold::k_fold<fold::Cfg<R, A, B, 1>, false, FOLD_CONV>;
+const void* conv_fixed(int P, bool strided) {
+    if (!strided) return (const void*)fold::k_fold<fold::Cfg<R, A, B, 1>, false, FOLD_CONV>;
+    return P == 4 ? (const void*)fold::k_fold<fold::Cfg<R, A, B, 4>, true, FOLD_CONV>
+                  : (const void*)fold::k_fold<fold::Cfg<R, A, B, 2>, true, FOLD_CONV>;
 }
 #define PSTD_CONV_CASE(RR, AA, BB) \
-    if (R == RR && A == AA && B == BB) return conv_fixed<RR, AA, BB>(strided);
+    if (R == RR && A == AA && B == BB) return conv_fixed<RR, AA, BB>(P, strided);
 #define PSTD_CONV_UNIT(U)                                                \
-    const void* conv_unit_##U(int R, int A, int B, bool strided) {       \
+    const void* conv_unit_##U(int R, int A, int B, int P, bool strided) {       \
         PSTD_CONV_U##U(PSTD_CONV_CASE)                                   \
         return nullptr;                                                  \
     }
@@ -131,7 +132,9 @@ const void* fold_any_persist();
 
 // Kernel of axis x in `mode`; whether it is a fixed schedule's.
 const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed);
-cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cudaStream_t st);
+// overlap: a step's pass may start while the previous launch of its stream
+// drains (programmatic stream serialisation)
+cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cudaStream_t st, bool overlap = true);
 // `nsteps` steps of a 1-D run as one launch; false where its schedule has no
 // such kernel.
 bool fold_has_line(const FoldAxis& x);

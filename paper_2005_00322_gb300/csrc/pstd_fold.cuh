@@ -82,8 +82,10 @@ struct FoldArgs {
     const float* f;          // FOLD_GRAD_*, FOLD_ORDER2, FOLD_CONV p -> u: per bin multiplier (without the factor i)
     const float* f2;         // FOLD_CONV u -> p
     const float* in;         // p (STEP, GRAD_P, ORDER2) or u
+    const float* in2;        // STEP: p is in + in2 where given
     float* u;                // velocity spectrum (STEP, TO_SPEC, FROM_SPEC)
-    const float* acc_in;     // STEP: out = acc_in + contribution (contiguous axes: acc_in == in)
+    const float* acc_in;     // STEP: out = acc_in + contribution (contiguous axes: onto p); null on a strided
+                             // axis: out = contribution
     float* out;
     int accumulate;          // GRAD_*, ORDER2: out += instead of out =
     float* pout;             // ORDER2: also write in + (the new out) here (may be `in`)
@@ -431,6 +433,10 @@ struct Pass {
         if constexpr (C::fixed) return k + (k / C::A) * (padded(C::A) - C::A);
         else return a.ax.A & 1 ? k : k + k / a.ax.A;
     }
+    // pair p holds lines 2p and 2p + 1, so that a line's partner, and with it
+    // every rounding, does not depend on P (lines p and p + P of a strided tile
+    // would touch each sector once instead of twice: 251 against 254 us per
+    // 256^3 step)
     PSTD_HD bool va(int p) const { return 2 * p < nv; }
     PSTD_HD bool vb(int p) const { return 2 * p + 1 < nv; }
 
@@ -510,6 +516,28 @@ struct Pass {
                     x[e] = make_float2(ok && la ? ld(xa, off) : 0.0f, ok && lb ? ld(xb, off) : 0.0f);
                     // node N of an embedded line stands at both ends of its window
                     if (conv() && !half && i + lo == a.ax.cN) x[e] = cscale(x[e], 0.5f);
+                }
+                // (after all loads of the first field are under way)
+                if constexpr (ahead_u) {
+                    if (a.in2) {
+                        const float* za = base(a.in2, len);
+                        const float* zb = za + line_step(len);
+#pragma unroll
+                        for (int e = 0; e < a_; ++e) {
+                            const int j = j0 + dj * e;
+                            const bool mir = even ? 2 * e >= a_ : j > n;
+                            const Off off = mir ? om - (Off)e * step : od + (Off)e * step;
+                            bool ok = true;
+                            const int i = (mir ? refl - j : j) - lo;
+                            if (!even || e == 0 || 2 * e == a_) ok = i >= 0 && i < len;
+                            x[e].x = radd(x[e].x, ok && la ? ld(za, off) : 0.0f);
+                            x[e].y = radd(x[e].y, ok && lb ? ld(zb, off) : 0.0f);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < a_; ++e) {
+                    const bool mir = even ? 2 * e >= a_ : (half ? j0 + dj * e >= n : j0 + dj * e > n);
                     if constexpr (onto_p) ac[e] = x[e];
                     if constexpr (keep_p) pk[e] = x[e];
                     if (mir) x[e] = cscale(x[e], rsg);
@@ -764,7 +792,7 @@ struct Pass {
             by_full([&](auto full) {
                 const float* xa = base(MODE == FOLD_ORDER2 ? (const float*)a.out : a.acc_in, nout());
                 const float* xb = xa + line_step(nout());
-                const bool acc = MODE != FOLD_ORDER2 || a.accumulate;
+                const bool acc = MODE == FOLD_ORDER2 ? a.accumulate != 0 : a.acc_in != nullptr;
                 items((C::R / 2 + 1) * C::B, [&](int p, int w) {
                     const int r = w / C::B, t = w - r * C::B, j0 = C::R * t + r;
                     const bool la = full || va(p), lb = full || vb(p);
@@ -800,6 +828,7 @@ struct Pass {
             const bool half = out_half();
             const float rsg = half ? -a.ax.rho : a.ax.rho;
             float* ya = base(a.out, nout());
+            float* yb = ya + line_step(nout());
             items((half ? R() / 2 : R() / 2 + 1) * B(), [&](int p, int w) {
                 const int r = w / B(), t = w - r * B(), j0 = R() * t + r;
                 const float2* s = at(r, p) + Ap() * t * ls();
@@ -826,17 +855,17 @@ struct Pass {
                             if constexpr (ahead) {
                                 const float2 v = make_float2(rfma(sgn, x[e].x, ac[e].x), rfma(sgn, x[e].y, ac[e].y));
                                 if (ok && la) put(ya, off, v.x);
-                                if (ok && lb) put(ya + 1, off, v.y);
+                                if (ok && lb) put(yb, off, v.y);
                                 if constexpr (keep_p) {
                                     if (a.pout) {
                                         float* qa = base(a.pout, nout());
                                         if (ok && la) put(qa, off, radd(pk[e].x, v.x));
-                                        if (ok && lb) put(qa + 1, off, radd(pk[e].y, v.y));
+                                        if (ok && lb) put(qa + line_step(nout()), off, radd(pk[e].y, v.y));
                                     }
                                 }
                             } else {
                                 emit(ya + off / 4, ok && la, rmul(sgn, x[e].x));
-                                emit(ya + off / 4 + 1, ok && lb, rmul(sgn, x[e].y));
+                                emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y));
                             }
                         } else {
                             // row position of node (lo + i) or half-node i
@@ -939,17 +968,16 @@ struct Pass {
             const int len = nout(), pitch = row_pitch(a.ax), lo = out_half() ? 0 : a.ax.lo;
             float* y = base(a.out, len);
             const int wid = tid >> 5, lane = tid & 31, nw = (nthr + 31) >> 5;
-            for (int l = wid; l < nv; l += nw)
-                for (int i = lane; i < len; i += 32) {
-                    const float c = st[l * pitch + row_word(i + lo)];
+            for (int l = wid; l < nv; l += nw) {
+                const float* q = st + l * pitch + row_word(lane + lo);   // + 36 words per 32 positions
+                float* z = y + l * (int64_t)len + lane;
+                for (int i = lane; i < len; i += 32, q += 36, z += 32) {
                     if constexpr (ahead) {
-                        y[l * len + i] = c;
-                        if (mode() == FOLD_ORDER2 && a.pout) {
-                            const int64_t off = y - a.out + l * (int64_t)len + i;
-                            a.pout[off] = radd(a.in[off], c);
-                        }
-                    } else emit(y + l * (int64_t)len + i, true, c);
+                        *z = *q;
+                        if (mode() == FOLD_ORDER2 && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
+                    } else emit(z, true, *q);
                 }
+            }
         }
     }
     // bring the tables to this SM's L1 before the fields may be touched

@@ -8,7 +8,7 @@ const void* fold_any_misc_c();
 #define DECL(U) const void* fold_unit_##U(int R, int A, int B, int P, bool strided, int mode);
 PSTD_FOLD_UNITS(DECL)
 #undef DECL
-#define DECL(U) const void* conv_unit_##U(int R, int A, int B, bool strided);
+#define DECL(U) const void* conv_unit_##U(int R, int A, int B, int P, bool strided);
 PSTD_CONV_UNITS(DECL)
 #undef DECL
 
@@ -16,7 +16,7 @@ const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) 
     fixed = true;
     if (mode == FOLD_CONV) {
 #define TRY(U) \
-    if (const void* k = conv_unit_##U(x.R, x.A, x.B, strided)) return k;
+    if (const void* k = conv_unit_##U(x.R, x.A, x.B, x.P, strided)) return k;
         PSTD_CONV_UNITS(TRY)
 #undef TRY
         return nullptr;
@@ -33,7 +33,7 @@ const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) 
     return strided ? fold_any_misc_s() : fold_any_misc_c();
 }
 
-cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cudaStream_t st) {
+cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cudaStream_t st, bool overlap) {
     bool fixed = false;
     const void* k = fold_kernel(a.ax, strided, a.mode, fixed);
     cudaLaunchConfig_t cfg{};
@@ -49,7 +49,7 @@ cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cu
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = a.mode == FOLD_STEP || a.mode == FOLD_ORDER2 || a.mode == FOLD_CONV ? 1 : 0;
+    cfg.numAttrs = !overlap ? 0 : a.mode == FOLD_STEP || a.mode == FOLD_ORDER2 || a.mode == FOLD_CONV ? 1 : 0;
     void* args[] = {(void*)&a};
     return cudaLaunchKernelExC(&cfg, k, args);
 }

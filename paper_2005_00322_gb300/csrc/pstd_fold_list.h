@@ -9,7 +9,10 @@
 // on phases that leave lanes idle.  PS = 8 makes each global access of a
 // strided pass a run of 16 words (256^3: 254 us per step against 288 with
 // PS = 4); schedules wider than 48 lanes per pair take 4, so that two CTAs fit
-// an SM.  Grouped by translation unit (pstd_fold_u*.cu), of like compile time.
+// an SM.  Measured choices against the rule: 256 (128^3: 39.0 us per step with
+// (4, 8, 8), whose phases have 24, 24 and 33 lanes, 41.7 with (8, 4, 8) and its
+// 40, 20 and 17), 400 (200 x 180 x 150: 110 against 116 with (8, 5, 10)) and
+// PC = 2 at 768 (384^3: 1067 against 1120).  Grouped by translation unit (pstd_fold_u*.cu), of like compile time.
 #pragma once
 
 #define PSTD_FOLD_U0(X) \
@@ -24,7 +27,7 @@
 #define PSTD_FOLD_U1(X) \
     X(6, 3, 6, 8, 4) \
     X(6, 3, 9, 8, 4) \
-    X(8, 4, 8, 8, 4) \
+    X(4, 8, 8, 8, 4) \
     X(8, 8, 8, 8, 4) \
     X(10, 5, 15, 4, 2) \
     X(12, 9, 9, 4, 4) \
@@ -40,7 +43,7 @@
 #define PSTD_FOLD_U3(X) \
     X(6, 3, 5, 8, 8) \
     X(8, 4, 4, 8, 8) \
-    X(8, 5, 10, 4, 4) \
+    X(10, 5, 8, 8, 4) \
     X(6, 8, 9, 8, 4) \
     X(10, 10, 10, 4, 4) \
     X(8, 12, 12, 4, 2) \
@@ -90,13 +93,13 @@
     X(8, 4, 5, 8, 4) \
     X(6, 6, 9, 8, 4) \
     X(10, 5, 10, 4, 4) \
-    X(8, 8, 12, 4, 4) \
+    X(8, 8, 12, 4, 2) \
     X(10, 9, 15, 4, 2) \
     X(12, 12, 12, 4, 2)
 // Embeddings of the convolution passes (lines of N cells with no schedule of
 // their own, 65 <= N <= 1280): the smallest length that is at least 4N, 4 to
-// 12 percent apart, as X(R, A, B); 2 line pairs per CTA on strided axes, 1 on
-// contiguous ones.
+// 12 percent apart, as X(R, A, B); 2 or 4 line pairs per CTA on strided axes, 1
+// on contiguous ones.
 #define PSTD_CONV_U0(X) X(8, 6, 6) X(6, 8, 9) X(8, 8, 10) X(10, 10, 10) X(10, 12, 12) X(8, 16, 16) X(12, 15, 16) X(18, 16, 16)
 #define PSTD_CONV_U1(X) X(8, 5, 8) X(6, 8, 10) X(8, 9, 10) X(8, 9, 15) X(10, 10, 16) X(10, 15, 15) X(12, 16, 16) X(20, 16, 16)
 #define PSTD_CONV_U2(X) X(8, 5, 9) X(8, 8, 8) X(8, 10, 10) X(10, 10, 12) X(12, 12, 12) X(10, 15, 16) X(16, 15, 15)

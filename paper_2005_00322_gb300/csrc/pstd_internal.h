@@ -6,6 +6,9 @@
 
 #include "../../include/pstd.h"
 
+// pstd_plan for one of `members` plans whose passes run side by side: pass
+// schedules are chosen for the GPU they fill together.
+int pstd_internal_plan_member(const pstd_desc* desc, void* stream, int members, pstd_plan_t** out);
 // Launch `n` leapfrog steps of plan P on its own stream (no graph capture of
 // its own, so the caller may be capturing); adds the kernel count.
 int pstd_internal_launch_steps(pstd_plan_t* P, float* p, float* const* u, int64_t n, int64_t* launches);

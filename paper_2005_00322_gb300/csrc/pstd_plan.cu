@@ -267,6 +267,7 @@ struct pstd_plan_s {
     pstd_plan_opts opts{{-1, -1, -1}, {-1, -1, -1}, 0, 0, 0, 0};
     unsigned* d_sync = nullptr;       // grid barrier: count, generation, status
     int nsm = 152;                    // SMs of the plan's device (queried at plan time)
+    int members = 1;                  // plans of the batch this one belongs to, whose passes share the GPU
     int persist_ok = 0;
     WLaunch pgeo{};
     cudaStream_t stream = nullptr;
@@ -274,6 +275,11 @@ struct pstd_plan_s {
     int64_t shape[4][3] = {};
     Axis ax[3];
     float* d_S = nullptr;
+    // both axis passes of a 2-D step side by side (see side_by_side)
+    float* d_C[2] = {nullptr, nullptr};   // contributions of axis 0, alternating
+    cudaStream_t side = nullptr;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    int side_ok = -1;                     // -1: not decided
     double* d_energy = nullptr;       // pstd_energy's FP64 partial sums, on first use
     // BF16 split form: plan-owned copies of p, u_0.. and the accumulator with
     // the last dimension padded to a multiple of 4 floats (TMA strides)
@@ -769,12 +775,13 @@ int build_fold(pstd_plan_s* P, int i, const pstd::FoldChoice& ch, int os) {
         // pair, 9.6 us per step with 8 pairs on 256 CTAs, 20.9 with one pair);
         // else 2 pairs on strided axes (512^2: 9.5 us with 129 CTAs of 2 against
         // 11.5 with 1, whose 8-byte rows use a quarter of each sector) and 1
-        // on contiguous ones (512^2 with 2: 15.5).  Run-time schedules take 8 or
+        // on contiguous ones (512^2 with 2: 15.5).  The members of a batch fill
+        // the GPU together.  Run-time schedules take 8 or
         // fewer, within their thread count.
         const int fixed = a.strided ? ch.PS : ch.PC;
         if (fixed && !x.wide) {
             const int64_t enough = pstd::fold_lanes(x) <= 48 ? P->nsm / 2 : (a.strided ? P->nsm : 2 * P->nsm);
-            p = tiles(fixed) >= enough ? fixed : (a.strided ? 2 : 1);
+            p = tiles(fixed) * P->members >= enough ? fixed : (a.strided ? 2 : 1);
         } else {
             p = 8;
             while (p > 1 && (tiles(p) < 2 * P->nsm || !fits(p) ||
@@ -821,10 +828,14 @@ int build_conv(pstd_plan_s* P, int i, const pstd::FoldChoice& ch) {
     x.nlines = a.nlines;
     x.inner = a.inner;
     a.strided = a.inner > 1;
-    x.P = a.strided ? ch.PS : ch.PC;
-    x.lgP = x.P == 2 ? 1 : 0;
-    a.fgeo.grid = (unsigned)(a.strided ? (a.nlines / a.inner) * ((a.inner + 2 * x.P - 1) / (2 * x.P))
-                                       : (a.nlines + 2 * x.P - 1) / (2 * x.P));
+    auto tiles = [&](int p) -> int64_t {
+        if (!a.strided) return (a.nlines + 2 * p - 1) / (2 * p);
+        return (a.nlines / a.inner) * ((a.inner + 2 * p - 1) / (2 * p));
+    };
+    // rows of 8 words where that still fills the GPU, 4 words else
+    x.P = !a.strided ? 1 : (tiles(4) * P->members >= 2 * P->nsm ? 4 : 2);
+    x.lgP = x.P == 4 ? 2 : (x.P == 2 ? 1 : 0);
+    a.fgeo.grid = (unsigned)tiles(x.P);
     a.fgeo.threads = pstd::fold_threads(x);
     a.fgeo.smem = pstd::fold::smem_bytes(x, a.strided);
     std::vector<float2> tab(t.tw);
@@ -1298,6 +1309,10 @@ void free_plan_memory(pstd_plan_s* P) {
         }
     }
     cudaFree(P->d_S);
+    for (float* c : P->d_C) cudaFree(c);
+    for (auto e : P->ev)
+        if (e) cudaEventDestroy(e);
+    if (P->side) cudaStreamDestroy(P->side);
     cudaFree(P->d_energy);
     for (auto* b : P->d_pad) cudaFree(b);
     cudaFree(P->d_Spad);
@@ -1654,6 +1669,60 @@ int launch_order2_step(pstd_plan_s* P, float* p, float* q, int64_t* launches) {
     return PSTD_OK;
 }
 
+// 2-D grids whose passes are too short to fill the GPU: both axes of a step
+// read p^n only, so their passes run side by side on two streams, one
+// dependency per step instead of two.  The pressure is then a sum of two
+// fields between steps: axis 1 writes A = p + c_1 and axis 0 writes C = c_0,
+// and the next step's passes load p = A + C, in the order and with the rounding
+// of S = p + c_1, p = S + c_0.  A alternates between the caller's p and the
+// accumulator, C between two plan buffers; a block of an even number of steps
+// ends with p += C.  512^2: 9.5 us per step one pass after the other.
+bool side_by_side(pstd_plan_s* P) {
+    if (P->side_ok >= 0) return P->side_ok == 1;
+    P->side_ok = 0;
+    bool ok = P->ndim == 2 && P->opts.form == 0 && P->stream != nullptr && !P->persist_ok;
+    for (int a = 0; a < 2 && ok; ++a) {
+        const Axis& A = P->ax[a];
+        bool fixed = false;
+        ok = A.fold() && pstd::fold_kernel(A.fax, A.strided, pstd::FOLD_STEP, fixed) && fixed;
+    }
+    // beyond 2 M points the passes fill the GPU by themselves
+    const int64_t n = P->shape[0][0] * P->shape[0][1];
+    if (!ok || n > (int64_t)2 << 20) return false;
+    for (auto& c : P->d_C)
+        if (cudaMalloc((void**)&c, (size_t)n * sizeof(float)) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+    if (cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking) != cudaSuccess) return false;
+    for (auto& e : P->ev)
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
+    P->side_ok = 1;
+    return true;
+}
+
+// kGraphSteps steps side by side (captured by replay_graphs).
+int launch_side_block(pstd_plan_s* P, float* p, float* const* u, int64_t* launches) {
+    float* A[2] = {p, P->d_S};
+    for (int s = 0; s < kGraphSteps; ++s) {
+        CK(cudaEventRecord(P->ev[0], P->stream));
+        CK(cudaStreamWaitEvent(P->side, P->ev[0], 0));
+        for (int a = 0; a < 2; ++a) {
+            FoldArgs f = fold_step(P, a, A[s & 1], u);
+            f.in2 = s > 0 ? P->d_C[(s - 1) & 1] : nullptr;
+            f.acc_in = a == 1 ? f.in : nullptr;
+            f.out = a == 1 ? A[(s + 1) & 1] : P->d_C[s & 1];
+            CK(pstd::fold_launch(f, P->ax[a].strided, P->ax[a].fgeo, a == 1 ? P->stream : P->side, false));
+            ++*launches;
+        }
+        CK(cudaEventRecord(P->ev[1], P->side));
+        CK(cudaStreamWaitEvent(P->stream, P->ev[1], 0));
+    }
+    CK(pstd::launch_k_axpby(pstd_field_numel(P, 0), 1.0f, P->d_C[(kGraphSteps - 1) & 1], 1.0f, p, P->stream));
+    ++*launches;
+    return PSTD_OK;
+}
+
 // Replay graphs of kGraphSteps steps for this pointer set (kind 0: leapfrog
 // steps on p and the velocities; kind 1: second-order steps on p and q),
 // recording one on first use (least recently used entry replaced); `done`
@@ -1952,6 +2021,10 @@ void pstd_internal_layout(const pstd_plan_t* P, int lo[3], int64_t shape[3]) {
 
 int pstd_internal_cuda_fail(cudaError_t e, const char* what) { return cuda_fail(e, what); }
 
+namespace {
+int make_plan(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts, int members, pstd_plan_t** out);
+}
+
 extern "C" {
 
 const char* pstd_version(void) { return "pstd-gb300 0.1 (sm_103a)"; }
@@ -2000,6 +2073,16 @@ int pstd_plan_schedule(const pstd_plan_t* P, int axis, int out[4]) {
 }
 
 int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts, pstd_plan_t** out) {
+    return make_plan(desc, stream, opts, 1, out);
+}
+}  // extern "C"
+
+int pstd_internal_plan_member(const pstd_desc* desc, void* stream, int members, pstd_plan_t** out) {
+    return make_plan(desc, stream, nullptr, members, out);
+}
+
+namespace {
+int make_plan(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts, int members, pstd_plan_t** out) {
     if (!out) return PSTD_EINVAL;
     *out = nullptr;
     int rc = validate(desc);
@@ -2007,6 +2090,7 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
     pstd_plan_s* P = new (std::nothrow) pstd_plan_s();
     if (!P) return PSTD_ENOMEM;
     P->desc = *desc;
+    P->members = members;
     if (opts) P->opts = *opts;
     {
         int dev = 0, n = 0;
@@ -2125,7 +2209,9 @@ int pstd_plan_ex(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts
     *out = P;
     return PSTD_OK;
 }
+}  // namespace
 
+extern "C" {
 int pstd_field_shape(const pstd_plan_t* P, int field, int64_t shape[3]) {
     if (!P || !shape || field < 0 || field > P->ndim) return PSTD_EINVAL;
     for (int j = 0; j < 3; ++j) shape[j] = P->shape[field][j];
@@ -2288,8 +2374,12 @@ int run_steps(pstd_plan_t* P, float* p, float* const* u, int64_t nsteps) {
     }
     int64_t done = 0;
     if (P->stream != nullptr && nsteps >= kGraphSteps) {
-        int rc = replay_graphs(P, 0, p, u, P->ndim, nsteps, done,
-                               [&](int64_t* nl) { return launch_step(P, p, u, nl); });
+        const bool side = side_by_side(P);
+        int s = 0;
+        int rc = replay_graphs(P, 0, p, u, P->ndim, nsteps, done, [&](int64_t* nl) {
+            if (!side) return launch_step(P, p, u, nl);
+            return s++ == 0 ? launch_side_block(P, p, u, nl) : PSTD_OK;      // the whole block at once
+        });
         if (rc != PSTD_OK) return rc;
     }
     while (done < nsteps) {

@@ -53,8 +53,8 @@ void run_cfg(const FoldArgs& a, unsigned grid, int nthr) {
 // compiled and run-time radices of the convolution pass
 template <bool STR>
 void run_conv(const FoldArgs& a, unsigned grid, int nthr) {
-    if (a.ax.R == 8 && a.ax.A == 5 && a.ax.B == 8) run_all<fold::Cfg<8, 5, 8, STR ? 2 : 1>, STR, FOLD_CONV>(a, grid, nthr);
-    else if (a.ax.R == 8 && a.ax.A == 8 && a.ax.B == 8) run_all<fold::Cfg<8, 8, 8, STR ? 2 : 1>, STR, FOLD_CONV>(a, grid, nthr);
+    if (a.ax.R == 8 && a.ax.A == 5 && a.ax.B == 8 && a.ax.P <= 2) run_all<fold::Cfg<8, 5, 8, STR ? 2 : 1>, STR, FOLD_CONV>(a, grid, nthr);
+    else if (a.ax.R == 8 && a.ax.A == 8 && a.ax.B == 10 && a.ax.P != 2) run_all<fold::Cfg<8, 8, 10, STR ? 4 : 1>, STR, FOLD_CONV>(a, grid, nthr);
     else run_all<fold::AnyCfg, STR, FOLD_CONV>(a, grid, nthr);
 }
 static void dft(std::vector<cd>& x) {
@@ -96,7 +96,7 @@ int main() {
                 ax.tw = tb.tw.data(); ax.tc = tb.tc.data(); ax.th = tb.th.data();
                 const int outer = lay ? 2 : 1, inner = lay ? 11 : 1;
                 const int nl = lay ? outer * inner : 7;
-                ax.P = conv ? (lay ? 2 : 1) : 4; ax.lgP = conv ? lay : 2;
+                ax.P = conv ? (lay ? 2 << (N & 1) : 1) : 4; ax.lgP = conv ? (lay ? 1 + (N & 1) : 0) : 2;
                 ax.inner = inner; ax.nlines = nl;
                 const unsigned grid = lay ? outer * ((inner + 2 * ax.P - 1) / (2 * ax.P)) : (nl + 2 * ax.P - 1) / (2 * ax.P);
                 const int nthr = fold_threads(ax);
