@@ -266,7 +266,7 @@ def hbm_case(peak: float, name: str = "cube256_ddnndd") -> dict:
     r.close()
     return {"workload": name, "ms_per_step": step_s * 1e3, "updates_per_s": cells(w) / step_s,
             "roofline": {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-                         "kernel": "k_wstep (fused axis pass)", "alg_bytes_per_launch": alg_step / w.ndim,
+                         "kernel": "k_fold (fused axis pass)", "alg_bytes_per_launch": alg_step / w.ndim,
                          "launch_s": per_launch}}
 
 
@@ -655,7 +655,7 @@ def main():
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "kernel": ("k_wgrad dir 4 (second-order axis pass)" if args.form == "order2"
-                           else "k_wstep (fused axis pass)") if single
+                           else "k_fold (fused axis pass)") if single
                 else "every member's axis passes (k_wstep register passes, k_step generic / convolution "
                      "passes), concurrent graph branches",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks else "fallback 6.8 TB/s",
