@@ -54,14 +54,22 @@ constexpr int cfg_blocks() {
 }
 constexpr int kAnyThreads = 384;
 
+// One axis pass on fixed radices.  Bound by latency: 256^3 (8, 8, 8) takes 84 to
+// 86 us a pass (160 to 250 us on the length-512 complex FFTs before), DRAM 31 to
+// 42%, issue 48 to 58%, L1 wavefronts 61% at 20 warps per SM; per point 36
+// floating-point, 20 (strided) or 30 (contiguous) integer and 15 memory
+// instructions.  Length 768 (8, 8, 12): 384^3 2.23 -> 1.08 ms per step.
+// Convolution passes (FOLD_CONV) are bound by instructions, four transforms of
+// 4N points and more per pair: 20 uneven 2-D grids 963 -> 300 us per step.
 template <class C, bool STR, int MODE>
 __global__ void __launch_bounds__(cfg_threads<C>(), cfg_blocks<C>()) k_fold(const __grid_constant__ FoldArgs a) {
     extern __shared__ float4 wsm4[];
     fold_pass<C, STR, MODE>(a, blockIdx.x, wsm4, threadIdx.x, blockDim.x);
 }
 // All steps of a 1-D run in one CTA: its one line pair is only ever touched by
-// this CTA, so a CTA barrier replaces the kernel boundary (line of 256 cells:
-// 2.4 us per step as separate launches) and p and the slots stay in its L1.
+// this CTA, so a CTA barrier replaces the kernel boundary and p and the slots
+// stay in its L1 (line of 256 cells: 2.4 us per step as separate launches, 2.1
+// here; bound by one CTA's chain of five phases).
 template <class C>
 __global__ void __launch_bounds__(cfg_threads<C>()) k_fold_line(const __grid_constant__ FoldArgs a, int64_t nsteps) {
 #ifdef __CUDA_ARCH__
@@ -72,6 +80,10 @@ __global__ void __launch_bounds__(cfg_threads<C>()) k_fold_line(const __grid_con
     }
 #endif
 }
+// Run-time radices: every phase holds a switch over them, so registers are those
+// of the largest (it spills above radix 10) and offsets are 64-bit; about three
+// times slower per point than fixed radices (224^3 477 us per step), still twice
+// as fast as the routes these lengths had (112 x 70: 57 -> 22 us).
 template <bool STR, int MODE>
 __global__ void __launch_bounds__(kAnyThreads, 2) k_fold_any(const __grid_constant__ FoldArgs a) {
     extern __shared__ float4 wsm4[];

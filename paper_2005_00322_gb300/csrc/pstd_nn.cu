@@ -344,8 +344,10 @@ __global__ void k_row_scale(const float* x, const float* sc, float* y, int64_t P
 // A CTA of 4 warps takes kMixX consecutive x of a sample and 128 y, the next
 // x's rows arriving (cp.async, second buffer) behind the current one's
 // products: lanes walk y (4 each, 32 apart, so shared reads and global accesses
-// are full lines), each warp has 8 output channels (12 shared reads feed 64
-// multiply-adds).
+// are full lines), each warp has 8 output channels.  256 samples of 32 channels
+// of 129 x 127 points: 0.44 ms a layer against 1.9 ms for the separate launches;
+// bound by shared-memory reads and issue (the multiply-adds alone are 0.17 ms,
+// the field's bytes 0.16 ms).
 constexpr int kMixC = 32, kMixK = 32, kMixX = 8, kMixY = 128;
 struct MixArgs {
     const float* W;
