@@ -84,8 +84,8 @@ struct FoldArgs {
     const float* in;         // p (STEP, GRAD_P, ORDER2) or u
     const float* in2;        // STEP: p is in + in2 where given
     float* u;                // velocity spectrum (STEP, TO_SPEC, FROM_SPEC)
-    const float* acc_in;     // STEP: out = acc_in + contribution (contiguous axes: onto p); null on a strided
-                             // axis: out = contribution
+    const float* acc_in;     // STEP: out = acc_in + contribution; null (fixed schedules only): out = contribution.
+                             // acc_in == in on contiguous lines: out = in (+ in2) + contribution
     float* out;
     int accumulate;          // GRAD_*, ORDER2: out += instead of out =
     float* pout;             // ORDER2: also write in + (the new out) here (may be `in`)
@@ -366,8 +366,9 @@ struct Pass {
     // Fixed schedules request what a phase needs from memory ahead of it, so
     // that the latency passes behind the barriers and the radices between:
     // the velocity slots after p1 (contiguous: before it), the accumulator
-    // after p3.  A contiguous leapfrog pass accumulates onto p itself, which
-    // p5's thread has read in p1; the second-order pass keeps that p for pout.
+    // after p3.  A contiguous leapfrog pass mostly accumulates onto p itself
+    // (acc_in == in, the last axis), which p5's thread has read in p1; the
+    // second-order pass keeps that p for pout.
     static constexpr bool ahead = C::fixed && (MODE == FOLD_STEP || MODE == FOLD_ORDER2 || MODE == FOLD_CONV);
     static constexpr bool ahead_u = C::fixed && MODE == FOLD_STEP;
     static constexpr bool onto_p = ahead_u && !STR;
@@ -788,7 +789,12 @@ struct Pass {
         return ok;
     }
     PSTD_HD void fetch_acc() {
-        if constexpr (ahead && !onto_p) {
+        if constexpr (ahead) {
+            // (contiguous lines of an axis that is not the last -- the later axes
+            // store one node -- add onto the accumulator like strided ones)
+            if constexpr (onto_p) {
+                if (a.acc_in == a.in) return;
+            }
             by_full([&](auto full) {
                 const float* xa = base(MODE == FOLD_ORDER2 ? (const float*)a.out : a.acc_in, nout());
                 const float* xb = xa + line_step(nout());
