@@ -2,7 +2,8 @@
 // accumulator it may be given -- p itself, another field, none -- and with the
 // pressure as one field or as a sum of two, on contiguous and strided lines,
 // against the run-time radices.  Prints the number of comparisons and of
-// failures; compiled and run by test_fold_forms_cpu.py.
+// failures, after the output of fold_emulation.cu's own run; compiled and run by
+// test_fold_forms_cpu.py.
 #define main emulation_main
 #include "fold_emulation.cu"
 #undef main
@@ -89,6 +90,7 @@ void all_forms() {
     }
 }
 int main() {
+    emulation_main();
     all_forms<8, 2, 3, 8, 8>();
     all_forms<6, 5, 9, 8, 4>();
     all_forms<4, 8, 8, 8, 4>();
