@@ -1101,20 +1101,22 @@ int build_axis(pstd_plan_s* P, int i) {
 
     // folded passes: every walled axis whose length has a schedule, unless the
     // caller asks for a register-FFT schedule
+    int os = P->opts.seqs_per_cta[i];
+    const int ov = P->opts.variant[i];
+    if (os == 0 || os > 256 || (os > 0 && (os & (os - 1)))) return PSTD_EINVAL;
     {
-        const int ov = P->opts.variant[i], os = P->opts.seqs_per_cta[i];
         pstd::FoldChoice ch{};
         const bool can = !a.periodic && !a.mid && a.L >= kFoldMinLength && pstd::fold_choose(a.L, ch);
         if (ov == kFold && !can) return PSTD_EINVAL;
         if (can && (ov == kFold || (ov < 0 && (os < 0 || pstd::wlanes(a.L) == 0)))) {
-            if (os == 0 || os > 256 || (os > 0 && (os & (os - 1)))) return PSTD_EINVAL;
             return build_fold(P, i, ch, ov == kFold ? os : -1);
         }
     }
 
     // lines with no schedule: the convolution on folded transforms, steps and
-    // first derivatives
-    if (a.kind == 2 && !a.periodic && !a.mid && P->opts.form == 0) {
+    // first derivatives (the register-FFT variants 1 to 5 do not exist there and
+    // are refused below)
+    if (a.kind == 2 && !a.periodic && !a.mid && P->opts.form == 0 && (ov < 1 || ov > 5)) {
         pstd::FoldChoice ch{};
         if (pstd::conv_choose(a.N, ch) && (int64_t)(a.N + 1) * a.inner < (int64_t)1 << 30) return build_conv(P, i, ch);
     }
@@ -1127,8 +1129,6 @@ int build_axis(pstd_plan_s* P, int i) {
     // the axis has enough lines to keep 2 CTAs per SM busy.
     int T = pstd::wlanes(a.L);
     int V = 0;
-    int os = P->opts.seqs_per_cta[i];
-    const int ov = P->opts.variant[i];
     // schedules 3, 4 and 5 are compiled for walled axes, L = 2 N (their
     // passes fix N = L / 2)
     if (ov == 5) {
@@ -1170,7 +1170,6 @@ int build_axis(pstd_plan_s* P, int i) {
         V = pstd::wlanes_v5(a.L) > 0 ? 5 : 4;
         T = V == 5 ? pstd::wlanes_v5(a.L) : pstd::wlanes_v4(a.L);
     }
-    if (os == 0 || os > 256 || (os > 0 && (os & (os - 1)))) return PSTD_EINVAL;
     const bool auto_os = os < 0;
     if (os < 0 && V >= 1 && T <= 128 && (a.nlines + 1) / 2 >= 2 * 2 * nsm) os = 2;
     // strided axes stage tiles of 2 os lines: 4 sequences make each staged
