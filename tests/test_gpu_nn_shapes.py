@@ -1,0 +1,46 @@
+"""Kernels of the learned operator over the shapes where their launch rules
+change, against FP64 on the same FP32 inputs.
+
+Tolerances: a fused multiply-add rounds once, 2^-24 of its result (2^-23 asked).
+"""
+import ctypes
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -24
+
+
+def lib():
+    from paper_2005_00322_gb300 import _abi
+    return _abi.load(), _abi
+
+
+def rnd(*shape, seed=0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randn(*shape, generator=g, device="cuda")
+
+
+def ptr(t):
+    return None if t is None else ctypes.c_void_p(t.data_ptr())
+
+
+def stream():
+    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+
+# all channels in a thread, groups with and without a remainder, one channel each; fewer points than threads
+@pytest.mark.parametrize("B,C,P", [(32, 32, 16383), (3, 7, 5000), (1, 32, 70000), (1, 20000, 16), (2, 1000, 257),
+                                   (1, 1, 400001), (65535, 1, 3), (1, 65535, 1)])
+def test_lift_and_its_adjoint(B, C, P):
+    L, _ = lib()
+    x, w, b = rnd(B, P, seed=1), rnd(C, seed=2), rnd(C, seed=3)
+    v = torch.full((B, C, P), 7.0, device="cuda")
+    assert L.pstd_nn_lift(ptr(x), ptr(w), ptr(b), ptr(v), B, C, P, stream()) == 0
+    want = w.double()[None, :, None] * x.double()[:, None, :] + b.double()[None, :, None]
+    assert ((v.double() - want).abs() <= 2 * EPS * want.abs()).all()
+    v.fill_(7.0)
+    assert L.pstd_nn_proj_bwd(ptr(x), ptr(w), ptr(v), B, C, P, stream()) == 0
+    want = w.double()[None, :, None] * x.double()[:, None, :]
+    assert ((v.double() - want).abs() <= 2 * EPS * want.abs()).all()
