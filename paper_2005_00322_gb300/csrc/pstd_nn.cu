@@ -170,8 +170,8 @@ __global__ void k_proj_bwd(const float* dout, const float* w, float* dv, int C, 
 }
 
 // Sums in FP64 run at a few operations per clock and SM, so a reduction is
-// spread over the GPU: kRed CTAs of one cluster each add up a share, and the
-// first adds the shares through distributed shared memory in a fixed order
+// spread over the GPU: the R <= kRed CTAs of one cluster each add up a share, and
+// the first adds the shares through distributed shared memory in a fixed order
 // (no workspace, no atomics, the same bits each time).
 constexpr int kRed = 8;
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -182,9 +182,9 @@ __device__ __forceinline__ unsigned cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 }
-// Sum over the cluster's CTAs of `acc` over their threads (256), valid in
+// Sum over the cluster's R CTAs of `acc` over their threads (256), valid in
 // thread 0 of rank 0.
-__device__ double cluster_sum(double acc) {
+__device__ double cluster_sum(double acc, unsigned R) {
     __shared__ double red[256];
     __shared__ double part;
     red[threadIdx.x] = acc;
@@ -198,7 +198,7 @@ __device__ double cluster_sum(double acc) {
     double tot = 0.0;
     if (cluster_rank() == 0 && threadIdx.x == 0) {
         const unsigned mine = (unsigned)__cvta_generic_to_shared(&part);
-        for (unsigned r = 0; r < kRed; ++r) {
+        for (unsigned r = 0; r < R; ++r) {
             unsigned at;
             double v;
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine), "r"(r));
@@ -211,18 +211,22 @@ __device__ double cluster_sum(double acc) {
 }
 
 // g[c] = sum_{b, i} x[b, c, i] * (y ? y[b, c or -, i] : 1); y indexed [b, i] when ybc == 0
-// One cluster of kRed CTAs per channel.  With one CTA per channel (32 of the
-// SMs) 32 channels of 32 x 16383 points took 138 us of FP64 adds alone.
+// One cluster of R CTAs per channel, which share out its samples (by_sample) or
+// the points of each.  With one CTA per channel (32 of the SMs) 32 channels of
+// 32 x 16383 points took 138 us of FP64 adds alone; with eight 4096 channels of
+// 64 points 209 us against 21, and the points of 16 samples of 1024 shared out
+// 29 us against 16.
 __global__ void __launch_bounds__(256) k_chan_dot(const float* x, const float* y, int ybc, float* g, int64_t B, int C,
-                                                  int64_t P) {
-    const int c = blockIdx.x / kRed;
+                                                  int64_t P, int R, int by_sample) {
+    const int c = blockIdx.x / R;
+    const int64_t rank = cluster_rank();
     // four independent chains of adds and loads per thread
     double acc[4] = {};
-    constexpr int64_t step = (int64_t)kRed * 256;
-    for (int64_t b = 0; b < B; ++b) {
+    const int64_t step = (by_sample ? 1 : R) * 256, i0 = (by_sample ? 0 : rank * 256) + threadIdx.x;
+    for (int64_t b = by_sample ? rank : 0; b < B; b += by_sample ? R : 1) {
         const float* xr = x + (b * C + c) * P;
         const float* yr = y ? (ybc ? y + (b * C + c) * P : y + b * P) : nullptr;
-        int64_t i = (int64_t)cluster_rank() * 256 + threadIdx.x;
+        int64_t i = i0;
         for (; i + 3 * step < P; i += 4 * step) {
             float xv[4], yv[4];
 #pragma unroll
@@ -235,8 +239,8 @@ __global__ void __launch_bounds__(256) k_chan_dot(const float* x, const float* y
         }
         for (; i < P; i += step) acc[0] += (double)xr[i] * (yr ? (double)yr[i] : 1.0);
     }
-    const double tot = cluster_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-    if (cluster_rank() == 0 && threadIdx.x == 0) g[c] = (float)tot;
+    const double tot = cluster_sum((acc[0] + acc[1]) + (acc[2] + acc[3]), R);
+    if (rank == 0 && threadIdx.x == 0) g[c] = (float)tot;
 }
 
 // out[j] = sum_b x[b, j] (sum over the leading dimension): a CTA takes 8
@@ -298,7 +302,7 @@ __global__ void __launch_bounds__(256) k_mse(const float* out, const float* targ
         acc += (double)df * (double)df;
         if (dout) dout[t] = s * df;
     }
-    const double tot = cluster_sum(acc);
+    const double tot = cluster_sum(acc, kRed);
     if (cluster_rank() == 0 && threadIdx.x == 0) loss[0] = (float)(tot / (double)n);
 }
 
@@ -464,16 +468,16 @@ __global__ void __launch_bounds__(128) k_mix(MixArgs a) {
     }
 }
 
-// Launch on clusters of kRed CTAs.
+// Launch on clusters of R CTAs.
 template <class... KA, class... CA>
-cudaError_t launch_cluster(void (*k)(KA...), unsigned grid, cudaStream_t st, CA... args) {
+cudaError_t launch_cluster(void (*k)(KA...), unsigned R, unsigned grid, cudaStream_t st, CA... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(256);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kRed;
+    at[0].val.clusterDim.x = R;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
@@ -620,8 +624,13 @@ int pstd_nn_proj_bwd(const float* dout, const float* w, float* dv, int64_t B, in
 int pstd_nn_chan_dot(const float* x, const float* y, int y_has_channels, float* g, int64_t B, int C, int64_t P,
                      void* stream) {
     if (!x || !g || C < 1 || B < 0 || P < 0 || C > 0x7fffffff) return PSTD_EINVAL;
-    if (C > 0x7fffffff / kRed) return PSTD_EINVAL;
-    return cuda_rc(launch_cluster(k_chan_dot, (unsigned)C * kRed, (cudaStream_t)stream, x, y, y_has_channels, g, B, C, P));
+    // eight CTAs per channel while the channels alone leave SMs idle and each
+    // share is worth a CTA; whole samples to a CTA where a sample's points would
+    // not give each thread four
+    const int R = C <= 2 * 152 && B * P >= 8192 ? kRed : 1;
+    const int by_sample = R > 1 && B >= R && P < 4 * 256 * R;
+    return cuda_rc(launch_cluster(k_chan_dot, R, (unsigned)C * R, (cudaStream_t)stream, x, y, y_has_channels, g, B, C,
+                                  P, R, by_sample));
 }
 
 int pstd_nn_sum_lead(const float* x, float* out, int64_t B, int64_t n, void* stream) {
@@ -641,7 +650,7 @@ int pstd_nn_adam(float* w, const float* g, float* m, float* v, int64_t n, float 
 
 int pstd_nn_mse(const float* out, const float* target, float* dout, float* loss, int64_t n, void* stream) {
     if (!out || !target || !loss || n < 1) return PSTD_EINVAL;
-    return cuda_rc(launch_cluster(k_mse, kRed, (cudaStream_t)stream, out, target, dout, loss, n));
+    return cuda_rc(launch_cluster(k_mse, kRed, kRed, (cudaStream_t)stream, out, target, dout, loss, n));
 }
 
 int pstd_nn_rel_err(const float* a, const float* ref, float* err, int64_t B, int64_t P, void* stream) {

@@ -44,3 +44,18 @@ def test_lift_and_its_adjoint(B, C, P):
     assert L.pstd_nn_proj_bwd(ptr(x), ptr(w), ptr(v), B, C, P, stream()) == 0
     want = w.double()[None, :, None] * x.double()[:, None, :]
     assert ((v.double() - want).abs() <= 2 * EPS * want.abs()).all()
+
+
+# one CTA a channel (few values, many channels), eight with whole samples or points shared out, tails of each
+@pytest.mark.parametrize("B,C,P", [(1, 4096, 64), (1, 304, 8192), (1, 305, 8192), (8, 3, 1024), (9, 2, 8191), (8, 2, 8192),
+                                   (7, 2, 2000), (100, 1, 83), (8191, 5, 1)])
+def test_channel_dots(B, C, P):
+    """The FP64 sums round once (2^-24 of the result, twice that asked)."""
+    L, _ = lib()
+    x, y = rnd(B, C, P, seed=1), rnd(B, C, P, seed=2)
+    g = torch.full((C,), 7.0, device="cuda")
+    for yy, ch in ((None, 0), (y, 1), (y[:, 0].contiguous(), 0)):
+        assert L.pstd_nn_chan_dot(ptr(x), ptr(yy), ch, ptr(g), B, C, P, stream()) == 0
+        prod = x.double() if yy is None else x.double() * (yy if ch else yy[:, None]).double()
+        want, mag = prod.sum(dim=(0, 2)), prod.abs().sum(dim=(0, 2))
+        assert ((g.double() - want).abs() <= 2 * EPS * want.abs() + 1e-14 * mag).all()
