@@ -59,3 +59,14 @@ def test_channel_dots(B, C, P):
         prod = x.double() if yy is None else x.double() * (yy if ch else yy[:, None]).double()
         want, mag = prod.sum(dim=(0, 2)), prod.abs().sum(dim=(0, 2))
         assert ((g.double() - want).abs() <= 2 * EPS * want.abs() + 1e-14 * mag).all()
+
+
+# either side of the rule (256 columns a row), rows and columns that fill no group
+@pytest.mark.parametrize("B,n", [(1, 255), (1, 256), (4, 1023), (4, 1024), (33, 7), (100, 25600), (100, 25599), (3, 400001)])
+def test_leading_sums(B, n):
+    """The FP64 sums round once (2^-24 of the result, twice that asked)."""
+    L, _ = lib()
+    x, out = rnd(B, n, seed=1), torch.full((n,), 7.0, device="cuda")
+    assert L.pstd_nn_sum_lead(ptr(x), ptr(out), B, n, stream()) == 0
+    want, mag = x.double().sum(0), x.double().abs().sum(0)
+    assert ((out.double() - want).abs() <= 2 * EPS * want.abs() + 1e-14 * mag).all()
