@@ -25,7 +25,7 @@ namespace {
 // thread) over 16-wide k slices staged in shared memory.  Tile shapes:
 // 64 x 64 for square-ish products, 256 x 16 / 16 x 256 for the tall or wide
 // products with a mode count (16) on one side, 16 x 16 for the small per-line
-// transforms, 32 x 32 for the channel-by-channel products (the weight gradients
+// transforms, 32 x 32 for many channel-by-channel products (the weight gradients
 // of 32 channels over 2048 chunks of 256 points: 152 us on 16 x 16 tiles).
 template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__(256) k_sgemm(pstd_gemm_desc d) {
@@ -531,7 +531,10 @@ int pstd_nn_gemm(const pstd_gemm_desc* d, void* stream) {
     const int64_t nb2 = d->batch2 > 1 ? d->batch2 : 1;
     if (nb2 > 1 && (d->K_last < 0 || d->K_last > d->K || (d->K_last > 0 && (!d->A || !d->B)))) return PSTD_EINVAL;
     if (d->batch * nb2 > 65535 || (d->M + 255) / 256 > 65535) return PSTD_EINVAL;
-    // the tile shape that computes the fewest padded outputs (ties: 64 x 64)
+    // The tile shape that computes the fewest padded outputs (ties: 64 x 64), the
+    // small tiles charged for their operand traffic: 1056 x 1056 x 256 takes 29 us on
+    // 64 x 64 tiles, 38 on 32 x 32.  32 x 32 tiles only where they fill the GPU (one
+    // product 32 x 32 x 1024: 27 us, 19 on four 16 x 16 tiles).
     static const int shapes[5][2] = {{64, 64}, {256, 16}, {16, 256}, {16, 16}, {32, 32}};
     int best = 0;
     int64_t best_cost = -1;
@@ -539,8 +542,9 @@ int pstd_nn_gemm(const pstd_gemm_desc* d, void* stream) {
         const int64_t bm = shapes[t][0], bn = shapes[t][1];
         const int64_t gm = (d->M + bm - 1) / bm;
         if (gm > 65535) continue;
-        // padded outputs, plus a charge for the extra operand traffic of thin tiles
-        const int64_t cost = gm * bm * ((d->N + bn - 1) / bn) * bn * (t == 3 ? 2 : 1);
+        const int64_t gn = (d->N + bn - 1) / bn;
+        if (t == 4 && gm * gn * d->batch * nb2 < 152) continue;
+        const int64_t cost = gm * bm * gn * bn * (t == 3 ? 4 : t == 4 ? 3 : 2);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = t; }
     }
     const cudaStream_t st = (cudaStream_t)stream;

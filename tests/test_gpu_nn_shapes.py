@@ -70,3 +70,18 @@ def test_leading_sums(B, n):
     assert L.pstd_nn_sum_lead(ptr(x), ptr(out), B, n, stream()) == 0
     want, mag = x.double().sum(0), x.double().abs().sum(0)
     assert ((out.double() - want).abs() <= 2 * EPS * want.abs() + 1e-14 * mag).all()
+
+
+# 64 x 64 against 32 x 32 tiles (ragged by up to half a tile), few and many small products
+@pytest.mark.parametrize("batch,M,N,K", [(1, 1056, 1056, 40), (1, 1031, 64, 33), (1, 96, 96, 17), (40, 96, 96, 17),
+                                         (151, 32, 32, 50), (152, 32, 32, 50), (38, 33, 40, 7), (1, 32, 32, 1024)])
+def test_product_tiles(batch, M, N, K):
+    """A sum of n products in FP32 is off by at most n half-ulps of the sum of
+    magnitudes, (n + 2) 2^-24 sum |a b|."""
+    L, abi = lib()
+    A, B, C = rnd(batch, M, K, seed=1), rnd(batch, K, N, seed=2), torch.full((batch, M, N), 7.0, device="cuda")
+    d = abi.PstdGemmDesc(batch, M, N, K, A.data_ptr(), M * K, K, 1, B.data_ptr(), K * N, N, 1, C.data_ptr(), M * N, N, 1,
+                         1.0, 0.0, 1, 0, 0, 0, K)
+    assert L.pstd_nn_gemm(ctypes.byref(d), stream()) == 0
+    want, mag = A.double() @ B.double(), A.double().abs() @ B.double().abs()
+    assert ((C.double() - want).abs() <= (K + 2) * EPS * mag).all()
