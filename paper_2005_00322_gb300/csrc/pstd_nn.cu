@@ -193,6 +193,7 @@ __device__ double cluster_sum(double acc, unsigned R) {
         if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
+    if (R == 1) return red[0];
     if (threadIdx.x == 0) part = red[0];
     cluster_sync();
     double tot = 0.0;
@@ -219,7 +220,7 @@ __device__ double cluster_sum(double acc, unsigned R) {
 __global__ void __launch_bounds__(256) k_chan_dot(const float* x, const float* y, int ybc, float* g, int64_t B, int C,
                                                   int64_t P, int R, int by_sample) {
     const int c = blockIdx.x / R;
-    const int64_t rank = cluster_rank();
+    const int64_t rank = R > 1 ? cluster_rank() : 0;
     // four independent chains of adds and loads per thread
     double acc[4] = {};
     const int64_t step = (by_sample ? 1 : R) * 256, i0 = (by_sample ? 0 : rank * 256) + threadIdx.x;
@@ -491,7 +492,7 @@ cudaError_t launch_cluster(void (*k)(KA...), unsigned R, unsigned grid, cudaStre
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = R > 1;
     return cudaLaunchKernelEx(&cfg, k, static_cast<KA>(args)...);
 }
 
