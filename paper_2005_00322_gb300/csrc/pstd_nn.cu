@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "pstd.h"
@@ -361,10 +362,12 @@ __global__ void k_row_scale(const float* x, const float* sc, float* y, int64_t P
 // here v is read and out written once.  Each sum runs in index order and they
 // are added last, so every value has the bits of the separate products (a relu
 // argument near zero keeps its sign).
-// A CTA of 4 warps takes kMixX consecutive x of a sample and 128 y, the next
+// A CTA of 4 warps takes nx <= kMixX consecutive x of a sample and 128 y, the next
 // x's rows arriving (cp.async, second buffer) behind the current one's
 // products: lanes walk y (4 each, 32 apart, so shared reads and global accesses
-// are full lines), each warp has 8 output channels.  256 samples of 32 channels
+// are full lines), each warp has 8 output channels.  A CTA whose y end within 32
+// or 64 takes 1 or 2 per lane, and warps beyond the channels only copy (4 channels
+// of 129 x 9 points, 256 samples, four layers: 708 us without either).  256 samples of 32 channels
 // of 129 x 127 points: 0.44 ms a layer against 1.9 ms for the separate launches;
 // bound by shared-memory reads and issue (the multiply-adds alone are 0.17 ms,
 // the field's bytes 0.16 ms).
@@ -379,26 +382,27 @@ struct MixArgs {
     const float* bias;
     const float* mask;
     float* out;
-    int C, X, Y, K, act;
+    int C, X, Y, K, act, nx;
 };
 __device__ __forceinline__ void copy4(float* dst, const float* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
 // acc[m][q] += sum_j cf[j][m] rows[j][q], j ascending
-__device__ __forceinline__ void mix_rows(float (&acc)[8][4], const float* cf, const float* rows, int n) {
+template <int Q>
+__device__ __forceinline__ void mix_rows(float (&acc)[8][Q], const float* cf, const float* rows, int n) {
     const float4* cp = (const float4*)cf;
 #pragma unroll 4
     for (int j = 0; j < n; ++j, rows += kMixY, cp += kMixC / 4) {
         const float4 c0 = cp[0], c1 = cp[1];
         const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-        float r[4];
+        float r[Q];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = rows[32 * q];
+        for (int q = 0; q < Q; ++q) r[q] = rows[32 * q];
 #pragma unroll
         for (int m = 0; m < 8; ++m)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[m][q] = fmaf(c[m], r[q], acc[m][q]);
+            for (int q = 0; q < Q; ++q) acc[m][q] = fmaf(c[m], r[q], acc[m][q]);
     }
 }
 inline size_t mix_smem(int C, int K) {
@@ -411,10 +415,10 @@ __global__ void __launch_bounds__(128) k_mix(MixArgs a) {
     float* const wc = tr + a.K * kMixY;                 // [C][32]: W of (input, output channel)
     float* const ac = wc + a.C * kMixC;                 // [2][K][32]: A of (mode, output channel)
     const int tid = threadIdx.x, lane = tid & 31, wrp = tid >> 5;
-    const int y0 = blockIdx.x * kMixY, x0 = blockIdx.y * kMixX;
+    const int y0 = blockIdx.x * kMixY, x0 = blockIdx.y * a.nx;
     const int ny = a.Y - y0 < kMixY ? a.Y - y0 : kMixY;
     const int64_t b = blockIdx.z, P = (int64_t)a.X * a.Y;
-    const int x1 = x0 + kMixX < a.X ? x0 + kMixX : a.X;
+    const int x1 = x0 + a.nx < a.X ? x0 + a.nx : a.X;
     auto issue = [&](int x, int buf) {
         float* d = vr + buf * a.C * kMixY;
         for (int i = wrp; i < a.C; i += 4) {
@@ -446,37 +450,45 @@ __global__ void __launch_bounds__(128) k_mix(MixArgs a) {
         const int k = t / kMixY, y = t % kMixY;
         tr[t] = y < ny ? a.T[k * a.sTk + (y0 + y) * a.sTy] : 0.0f;
     }
-    for (int x = x0; x < x1; ++x) {
-        const int buf = (x - x0) & 1;
-        if (x + 1 < x1) {
-            issue(x + 1, buf ^ 1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncthreads();
-        float aw[8][4] = {}, as[8][4] = {};
-        mix_rows(as, ac + buf * a.K * kMixC + wrp * 8, tr + lane, a.K);
-        mix_rows(aw, wc + wrp * 8, vr + buf * a.C * kMixY + lane, a.C);
-        __syncthreads();                       // this buffer may be refilled
+    auto rows = [&](auto nq) {
+        constexpr int Q = decltype(nq)::value;
+        for (int x = x0; x < x1; ++x) {
+            const int buf = (x - x0) & 1;
+            if (x + 1 < x1) {
+                issue(x + 1, buf ^ 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            float aw[8][Q] = {}, as[8][Q] = {};
+            if (wrp * 8 < a.C) {
+                mix_rows<Q>(as, ac + buf * a.K * kMixC + wrp * 8, tr + lane, a.K);
+                mix_rows<Q>(aw, wc + wrp * 8, vr + buf * a.C * kMixY + lane, a.C);
+            }
+            __syncthreads();                       // this buffer may be refilled
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int o = wrp * 8 + m;
-            if (o >= a.C) break;
-            const int64_t off = (b * a.C + o) * P + (int64_t)x * a.Y + y0;
-            const float bv = a.bias ? a.bias[o] : 0.0f;
+            for (int m = 0; m < 8; ++m) {
+                const int o = wrp * 8 + m;
+                if (o >= a.C) break;
+                const int64_t off = (b * a.C + o) * P + (int64_t)x * a.Y + y0;
+                const float bv = a.bias ? a.bias[o] : 0.0f;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int y = lane + 32 * q;
-                if (y >= ny) continue;
-                float z = aw[m][q] + as[m][q];
-                if (a.bias) z += bv;
-                if (a.act == 1) z = fmaxf(z, 0.0f);
-                if (a.mask && a.mask[off + y] <= 0.0f) z = 0.0f;
-                a.out[off + y] = z;
+                for (int q = 0; q < Q; ++q) {
+                    const int y = lane + 32 * q;
+                    if (y >= ny) continue;
+                    float z = aw[m][q] + as[m][q];
+                    if (a.bias) z += bv;
+                    if (a.act == 1) z = fmaxf(z, 0.0f);
+                    if (a.mask && a.mask[off + y] <= 0.0f) z = 0.0f;
+                    a.out[off + y] = z;
+                }
             }
         }
-    }
+    };
+    if (ny <= 32) rows(std::integral_constant<int, 1>{});
+    else if (ny <= 64) rows(std::integral_constant<int, 2>{});
+    else rows(std::integral_constant<int, 4>{});
 }
 
 // Launch on clusters of R CTAs.
@@ -586,7 +598,12 @@ int pstd_nn_mix(const float* W, int w_transposed, const float* v, const float* A
     a.Y = Y;
     a.K = K;
     a.act = act;
-    const dim3 grid((unsigned)((Y + kMixY - 1) / kMixY), (unsigned)((X + kMixX - 1) / kMixX), (unsigned)B);
+    // eight x per CTA share its copy of W and T; fewer where that leaves SMs idle
+    // (one sample of 32 channels of 129 x 127 points: 17 CTAs)
+    const int64_t ny = (Y + kMixY - 1) / kMixY;
+    a.nx = kMixX;
+    while (a.nx > 1 && ny * ((X + a.nx - 1) / a.nx) * B < 2 * 152) a.nx /= 2;
+    const dim3 grid((unsigned)ny, (unsigned)((X + a.nx - 1) / a.nx), (unsigned)B);
     const size_t smem = mix_smem(C, K);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_mix, cudaFuncAttributeMaxDynamicSharedMemorySize,

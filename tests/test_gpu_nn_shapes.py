@@ -85,3 +85,30 @@ def test_product_tiles(batch, M, N, K):
     assert L.pstd_nn_gemm(ctypes.byref(d), stream()) == 0
     want, mag = A.double() @ B.double(), A.double().abs() @ B.double().abs()
     assert ((C.double() - want).abs() <= (K + 2) * EPS * mag).all()
+
+
+# 1, 2 and 4 points a lane, in the last and in the only tile; channels that leave warps idle; 8, 4 and 1 rows a CTA
+@pytest.mark.parametrize("B,C,X,Y", [(3, 32, 17, 32), (3, 9, 17, 33), (2, 8, 9, 64), (2, 16, 9, 65), (1, 5, 5, 160),
+                                     (1, 24, 5, 192), (1, 4, 5, 193), (304, 2, 9, 10), (40, 3, 37, 20), (1, 32, 129, 127)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_mix_rows(B, C, X, Y, adjoint):
+    """A layer's second half, bit for bit the separate products (sums in index
+    order, added last) followed by bias and relu, or by the mask."""
+    L, abi = lib()
+    K, P = 7, X * Y
+    W, v, A, T = rnd(C, C, seed=1), rnd(B, C, X, Y, seed=2), rnd(B, C, X, K, seed=3), rnd(K, Y, seed=4)
+    bias, mask = (None, rnd(B, C, X, Y, seed=5)) if adjoint else (rnd(C, seed=5), None)
+    out = torch.full_like(v, 7.0)
+    assert L.pstd_nn_mix(ptr(W), int(adjoint), ptr(v), ptr(A), ptr(T), 1, ptr(bias), ptr(mask), ptr(out), B, C, X, Y, K,
+                         0 if adjoint else 1, stream()) == 0
+
+    def product(batch, M, N, K, A, sA, Bm, sB):
+        o = torch.empty(batch * M * N, device="cuda")
+        d = abi.PstdGemmDesc(batch, M, N, K, A.data_ptr(), *sA, Bm.data_ptr(), *sB, o.data_ptr(), M * N, N, 1, 1.0, 0.0, 1,
+                             0, 0, 0, K)
+        assert L.pstd_nn_gemm(ctypes.byref(d), stream()) == 0
+        return o.view(B, C, X, Y)
+    z = (product(B, C, P, C, W, (0, 1, C) if adjoint else (0, C, 1), v, (C * P, P, 1))
+         + product(1, B * C * X, Y, K, A, (0, K, 1), T, (0, Y, 1)))
+    want = torch.where(mask > 0, z, torch.zeros_like(z)) if adjoint else torch.relu(z + bias[None, :, None, None])
+    assert torch.equal(out, want)
