@@ -241,7 +241,9 @@ __global__ void __launch_bounds__(256) k_chan_dot(const float* x, const float* y
         }
         for (; i < P; i += step) acc[0] += (double)xr[i] * (yr ? (double)yr[i] : 1.0);
     }
-    const double tot = cluster_sum((acc[0] + acc[1]) + (acc[2] + acc[3]), R);
+    // (rows too short for the unrolled loop skip the additions of its chains)
+    const double own = 3 * step < P ? (acc[0] + acc[1]) + (acc[2] + acc[3]) : acc[0];
+    const double tot = cluster_sum(own, R);
     if (rank == 0 && threadIdx.x == 0) g[c] = (float)tot;
 }
 
