@@ -22,11 +22,11 @@ struct FoldLaunch {
 // schedule (a step's axis passes, last axis first, a grid barrier after each).
 struct FoldPersistArgs {
     FoldArgs ax[3];
-    int strided[3];
     unsigned items[3];
     int ndim;
     int64_t nsteps;
     GridSync sync;
+    unsigned tables;         // > 0: a plan's tables are copied to this offset (bytes) of shared memory
     int members;             // > 0: a batch, passes and prefix sums in device memory
     const FoldArgs* mem;     // [members][3]
     const int64_t* prefix;   // [3][members + 1]
@@ -90,10 +90,109 @@ __global__ void __launch_bounds__(kAnyThreads, 2) k_fold_any(const __grid_consta
     fold_pass<AnyCfg, STR, MODE>(a, blockIdx.x, wsm4, threadIdx.x, blockDim.x);
 }
 
+// A whole run as one cooperative kernel (grid and barrier as in
+// pstd_persist.cuh), for one plan or a batch: CS and CC are the passes of
+// strided and contiguous lines.  Bound by the barrier's round trips (about 3 us a
+// pass) and a pass' own chain.  Per step, against run-time radices for every
+// length, and the register FFTs before: 512^2 15.4, 42.7, 18.1 us; 256^2 11.6, 29.7,
+// 11.3; 128^3 62, 161, 107; 256^3 422, 805, 622; a line of 256 cells 3.1, 11.4, 4.3.
+template <class CS, class CC>
+constexpr int persist_threads() {
+    if (!CS::fixed) return kAnyThreads;
+    const int s = cfg_threads<CS>(), c = cfg_threads<CC>();
+    return s > c ? s : c;
+}
+template <class CS, class CC>
+constexpr int persist_blocks() {
+    if (!CS::fixed) return 2;
+    // 32 registers above cfg_blocks' for the loops and the two passes' addresses
+    constexpr int m = CS::R > CS::A ? CS::R : CS::A, b = 65536 / ((4 * m + 96) * persist_threads<CS, CC>());
+    return b > 8 ? 8 : (b >= 2 ? b : (m <= 10 && persist_threads<CS, CC>() * 2 * 96 <= 65536 ? 2 : 1));
+}
+template <class CS, class CC>
+__global__ void __launch_bounds__(persist_threads<CS, CC>(), persist_blocks<CS, CC>())
+    k_fold_persist(const __grid_constant__ FoldPersistArgs a) {
+#ifdef __CUDA_ARCH__
+    extern __shared__ float4 wsm4[];
+    // The passes' arguments in shared memory: through a reference into the
+    // parameters or global memory every field is a load of its own (a line of 256
+    // cells: 7.9 us per step).  A batch keeps each pass' last member, which for a
+    // CTA of one item per pass is found and fetched once a run.
+    __shared__ FoldArgs args[3];
+    auto fetch = [&](FoldArgs& d, const FoldArgs& src) {
+        for (int i = threadIdx.x; i < (int)(sizeof(FoldArgs) / 4); i += blockDim.x)
+            ((int*)&d)[i] = ((const int*)&src)[i];
+    };
+    __shared__ int64_t items[3];
+    __shared__ int first[3], own[3];     // members of the first item and of args[k]
+    if (!a.members)
+        for (int k = 0; k < a.ndim; ++k) fetch(args[k], a.ax[a.ndim - 1 - k]);
+    if (threadIdx.x < a.ndim) {
+        const int k = threadIdx.x;
+        const int64_t* pre = a.prefix + (size_t)k * (a.members + 1);
+        items[k] = a.members ? pre[a.members] : (int64_t)a.items[a.ndim - 1 - k];
+        first[k] = a.members && blockIdx.x < items[k] ? member_of(pre, a.members, blockIdx.x) : 0;
+        own[k] = -1;
+    }
+    __syncthreads();
+    // A barrier's acquire empties L1, so tables read through it arrive from L2 in
+    // every pass (256^2: 15.8 us per step).
+    if (a.tables) {
+        char* to = (char*)wsm4 + a.tables;
+        auto keep = [&](const float2*& t, int n) {
+            for (int i = threadIdx.x; i < n; i += blockDim.x) ((float2*)to)[i] = t[i];
+            __syncthreads();
+            if (threadIdx.x == 0) t = (const float2*)to;
+            to += n * sizeof(float2);
+        };
+        for (int k = 0; k < a.ndim; ++k) {
+            FoldAxis& x = args[k].ax;
+            keep(x.tw, x.M);
+            keep(x.tc, x.R / 2 * x.nk);
+            keep(args[k].coef, 2 * (x.N + 1));
+        }
+        __syncthreads();
+    }
+    unsigned gen = threadIdx.x == 0 ? ld_acquire(a.sync.gen) : 0;
+    for (int64_t s = 0; s < a.nsteps; ++s) {
+        for (int k = 0; k < a.ndim; ++k) {
+            const int64_t* pre = a.prefix + (size_t)k * (a.members + 1);
+            const int64_t n = items[k];
+            for (int64_t it = blockIdx.x; it < n; it += gridDim.x) {
+                unsigned item = (unsigned)it;
+                if (a.members) {
+                    const int m = it == blockIdx.x ? first[k] : member_of(pre, a.members, it);
+                    item = (unsigned)(it - pre[m]);
+                    if (m != own[k]) {
+                        __syncthreads();         // (every thread has read own)
+                        fetch(args[k], a.mem[(size_t)m * 3 + k]);
+                        if (threadIdx.x == 0) own[k] = m;
+                        __syncthreads();
+                    }
+                }
+                const FoldArgs& w = args[k];
+                if (w.ax.inner > 1) fold_pass<Resident<CS>, true, FOLD_STEP>(w, item, wsm4, threadIdx.x, blockDim.x);
+                else fold_pass<Resident<CC>, false, FOLD_STEP>(w, item, wsm4, threadIdx.x, blockDim.x);
+                __syncthreads();     // shared memory is reused by the next item
+            }
+            if (!grid_sync(a.sync, gen)) return;
+        }
+    }
+#endif
+}
+
 }  // namespace fold
 
-// Kernel of a schedule (mode FOLD_STEP, FOLD_ORDER2 or FOLD_LINE) with P pairs
-// per CTA, or null where it is not compiled; one function per translation unit.
+// Lengths 2^k and 3 2^k: those that had kernels of every kind on the register
+// FFTs.  Their cooperative run has a form for many lines too (the form for few, 2
+// and 1 pairs, took 807 us per 256^3 step and 145 per 128^3 step).
+constexpr bool fold_dyadic(int L) {
+    while (L % 2 == 0) L /= 2;
+    return L == 1 || L == 3;
+}
+// Kernel of a schedule (mode FOLD_STEP, FOLD_ORDER2, FOLD_LINE or FOLD_PERSIST)
+// with P pairs per CTA, or null where it is not compiled; one function per
+// translation unit.
 template <class C, bool STR>
 const void* fold_mode(int mode) {
     if (mode == FOLD_STEP) return (const void*)fold::k_fold<C, STR, FOLD_STEP>;
@@ -102,6 +201,12 @@ const void* fold_mode(int mode) {
 }
 template <int R, int A, int B, int PS, int PC>
 const void* fold_fixed(int P, bool strided, int mode) {
+    if (mode == FOLD_PERSIST) {
+        if (P == 1) return (const void*)fold::k_fold_persist<fold::Cfg<R, A, B, 2>, fold::Cfg<R, A, B, 1>>;
+        if constexpr (fold_dyadic(R * A * B))
+            return (const void*)fold::k_fold_persist<fold::Cfg<R, A, B, PS>, fold::Cfg<R, A, B, PC>>;
+        return nullptr;
+    }
     if (mode == FOLD_LINE) return P == 1 && !strided ? (const void*)fold::k_fold_line<fold::Cfg<R, A, B, 1>> : nullptr;
     if (strided) {
         if (P == PS) return fold_mode<fold::Cfg<R, A, B, PS>, true>(mode);
@@ -139,7 +244,8 @@ const void* conv_fixed(int P, bool strided) {
 // pstd_fold_any*.cu: the run-time schedules.  mode < 0: one kernel for the
 // derivative, conversion and second-order modes.
 const void* fold_any_step(bool strided);
-const void* fold_any_misc(bool strided);
+const void* fold_any_misc_s();
+const void* fold_any_misc_c();
 const void* fold_any_persist();
 
 // Kernel of axis x in `mode`; whether it is a fixed schedule's.
@@ -151,6 +257,22 @@ cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cu
 // such kernel.
 bool fold_has_line(const FoldAxis& x);
 cudaError_t fold_launch_line(const FoldArgs& a, int64_t nsteps, const FoldLaunch& g, cudaStream_t st);
+// The cooperative kernel of an axis and its CTA.  Compiled schedules (`fixed`)
+// run 2 line pairs per CTA on strided lines and 1 on contiguous ones or, where
+// `many` is set and compiled, the schedule's own PS and PC; the run-time one the
+// plan's pairs.
+struct FoldPersist {
+    const void* kernel;
+    int threads;
+    bool fixed;
+    int PS, PC;
+};
+FoldPersist fold_persist(const FoldAxis& x, bool many, int PS, int PC);
+// CTAs of a pass with p line pairs each
+inline int64_t fold_tiles(const FoldAxis& x, bool strided, int p) {
+    if (!strided) return (x.nlines + 2 * p - 1) / (2 * p);
+    return (x.nlines / x.inner) * ((x.inner + 2 * p - 1) / (2 * p));
+}
 // Raise the dynamic shared-memory limit of the kernels of axis x.
 cudaError_t fold_set_smem(const FoldAxis& x, bool strided, int bytes);
 

@@ -73,7 +73,8 @@ struct FoldAxis {
 
 enum { FOLD_STEP = 0, FOLD_GRAD_P = 1, FOLD_GRAD_U = 2, FOLD_TO_SPEC = 3, FOLD_FROM_SPEC = 4, FOLD_ORDER2 = 5,
        FOLD_CONV = 7,        // leapfrog pass of an embedded line: p -> u, u += , u -> p, p +=
-       FOLD_LINE = 6 };        // FOLD_LINE: the kernel that loops over FOLD_STEP passes of a 1-D run
+       // kernels that loop over FOLD_STEP passes: a 1-D run, a cooperative run
+       FOLD_LINE = 6, FOLD_PERSIST = 8 };
 
 struct FoldArgs {
     FoldAxis ax;
@@ -264,8 +265,14 @@ template <int R_, int A_, int B_, int P_>
 struct Cfg {
     static constexpr int R = R_, A = A_, B = B_, P = P_;
     static constexpr bool fixed = R_ > 0;
+    static constexpr bool resident = false;
 };
 using AnyCfg = Cfg<0, 0, 0, 0>;
+// tables that may lie in shared memory (a cooperative run's)
+template <class C>
+struct Resident : C {
+    static constexpr bool resident = true;
+};
 
 PSTD_HD int padded(int A) { return A | 1; }   // odd stride of k2 / t: no bank conflicts between lanes
 PSTD_HD int sub_words(int A, int B) { return padded(A) * B; }
@@ -377,6 +384,7 @@ struct Pass {
     float2 ac[ahead ? C::A : 1];
     float2 pk[keep_p ? C::A : 1];
 
+    static PSTD_HD float2 tab(const float2* p) { if constexpr (C::resident) return *p; else return ldc2(p); }
     PSTD_HD int R() const { if constexpr (C::fixed) return C::R; else return a.ax.R; }
     PSTD_HD int A() const { if constexpr (C::fixed) return C::A; else return a.ax.A; }
     PSTD_HD int B() const { if constexpr (C::fixed) return C::B; else return a.ax.B; }
@@ -548,7 +556,7 @@ struct Pass {
                 float2* d = at(r, p) + Ap() * t * ls();
 #pragma unroll
                 for (int k = 0; k < a_; ++k) {
-                    if (k > 0 || a.ax.g) x[k] = cmul(x[k], ldc2(&a.ax.tw[k * B() + t]));
+                    if (k > 0 || a.ax.g) x[k] = cmul(x[k], tab(&a.ax.tw[k * B() + t]));
                     d[k * ls()] = x[k];
                 }
             });
@@ -659,7 +667,7 @@ struct Pass {
                     if (in_half<PM>()) {
 #pragma unroll
                         for (int r = 0; r < H; ++r) {
-                            const float2 t = ldc2(&a.ax.th[r * nk + k]);
+                            const float2 t = tab(&a.ax.th[r * nk + k]);
                             w[r] = cmul(s[r * rs + lk], t);
                             w[r_ - 1 - r] = cscale(cmulc(s[r * rs + lkb], t), -sg);
                         }
@@ -667,11 +675,11 @@ struct Pass {
                         w[0] = s[lk];
 #pragma unroll
                         for (int r = 1; r < H; ++r) {
-                            const float2 t = ldc2(&a.ax.tc[(r - 1) * nk + k]);
+                            const float2 t = tab(&a.ax.tc[(r - 1) * nk + k]);
                             w[r] = cmul(s[r * rs + lk], t);
                             w[r_ - r] = cscale(cmulc(s[r * rs + lkb], t), sg);
                         }
-                        w[H] = cmul(s[H * rs + lk], ldc2(&a.ax.tc[(H - 1) * nk + k]));
+                        w[H] = cmul(s[H * rs + lk], tab(&a.ax.tc[(H - 1) * nk + k]));
                     }
                     Dft<r_, false>::run(w);
                     if (in_half<PM>()) half_twiddle<r_, false>(w, std::make_integer_sequence<int, r_>{});
@@ -721,7 +729,7 @@ struct Pass {
                     Dft<r_, true>::run(w);
 #pragma unroll
                     for (int r = 0; r < H; ++r) {
-                        const float2 t = ldc2(&a.ax.th[r * nk + k]);
+                        const float2 t = tab(&a.ax.th[r * nk + k]);
                         s[r * rs + lk] = cmulc(w[r], t);
                         if (k != kb) s[r * rs + lkb] = cscale(cmul(w[r_ - 1 - r], t), -sg);
                     }
@@ -731,11 +739,11 @@ struct Pass {
                     if (k != kb) s[lkb] = cscale(w[0], sg);
 #pragma unroll
                     for (int r = 1; r < H; ++r) {
-                        const float2 t = ldc2(&a.ax.tc[(r - 1) * nk + k]);
+                        const float2 t = tab(&a.ax.tc[(r - 1) * nk + k]);
                         s[r * rs + lk] = cmulc(w[r], t);
                         if (k != kb) s[r * rs + lkb] = cscale(cmul(w[r_ - r], t), sg);
                     }
-                    const float2 t = ldc2(&a.ax.tc[(H - 1) * nk + k]);
+                    const float2 t = tab(&a.ax.tc[(H - 1) * nk + k]);
                     s[H * rs + lk] = cmulc(w[H], t);
                     if (k != kb) s[H * rs + lkb] = cscale(cmul(w[H], t), sg);
                 }
@@ -756,7 +764,7 @@ struct Pass {
         for (int q = 0; q < r_; ++q) {
             // outputs q >= R/2 take the coefficients times sg (the second half
             // of the table)
-            const float2 cf = ldc2(&a.coef[bin(k, q) + (2 * q < r_ ? 0 : N() + 1)]);
+            const float2 cf = tab(&a.coef[bin(k, q) + (2 * q < r_ ? 0 : N() + 1)]);
             const float2 v = make_float2(rfma(cf.x, w[q].x, uv[q].x), rfma(cf.x, w[q].y, uv[q].y));
             store_slot(sl, k, kb, q, v);
             w[q] = cscale(v, cf.y);
@@ -842,7 +850,7 @@ struct Pass {
 #pragma unroll
                 for (int k = 0; k < a_; ++k) {
                     x[k] = s[k * ls()];
-                    if (k > 0 || a.ax.g) x[k] = cmulc(x[k], ldc2(&a.ax.tw[k * B() + t]));
+                    if (k > 0 || a.ax.g) x[k] = cmulc(x[k], tab(&a.ax.tw[k * B() + t]));
                 }
                 Dft<a_, true>::run(x);
                 if (a.ax.g) half_twiddle<a_, true>(x, std::make_integer_sequence<int, a_>{});
@@ -915,7 +923,7 @@ struct Pass {
 #pragma unroll
                 for (int k = 0; k < a_; ++k) {
                     x[k] = s[k * ls()];
-                    if (k > 0) x[k] = cmulc(x[k], ldc2(&a.ax.tw[k * B() + t]));
+                    if (k > 0) x[k] = cmulc(x[k], tab(&a.ax.tw[k * B() + t]));
                 }
                 Dft<a_, true>::run(x);
 #pragma unroll
@@ -939,7 +947,7 @@ struct Pass {
                 Dft<a_, false>::run(x);
 #pragma unroll
                 for (int k = 0; k < a_; ++k) {
-                    if (k > 0) x[k] = cmul(x[k], ldc2(&a.ax.tw[k * B() + t]));
+                    if (k > 0) x[k] = cmul(x[k], tab(&a.ax.tw[k * B() + t]));
                     s[k * ls()] = x[k];
                 }
             });
@@ -989,6 +997,9 @@ struct Pass {
     // bring the tables to this SM's L1 before the fields may be touched
     PSTD_HD void warm() const {
 #ifdef __CUDA_ARCH__
+        if constexpr (C::resident) {
+            if (__isShared(a.ax.tw)) return;
+        }
         auto touch = [&](const void* p, int bytes) {
             for (int i = tid * 128; i < bytes; i += nthr * 128)
                 asm volatile("prefetch.global.L1 [%0];" ::"l"((const char*)p + i));

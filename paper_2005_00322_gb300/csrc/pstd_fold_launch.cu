@@ -3,8 +3,6 @@
 
 namespace pstd {
 
-const void* fold_any_misc_s();
-const void* fold_any_misc_c();
 #define DECL(U) const void* fold_unit_##U(int R, int A, int B, int P, bool strided, int mode);
 PSTD_FOLD_UNITS(DECL)
 #undef DECL
@@ -21,7 +19,7 @@ const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) 
 #undef TRY
         return nullptr;
     }
-    if (!x.wide && (mode == FOLD_STEP || mode == FOLD_ORDER2 || mode == FOLD_LINE)) {
+    if (!x.wide && (mode == FOLD_STEP || mode == FOLD_ORDER2 || mode == FOLD_LINE || mode == FOLD_PERSIST)) {
 #define TRY(U) \
     if (const void* k = fold_unit_##U(x.R, x.A, x.B, x.P, strided, mode)) return k;
         PSTD_FOLD_UNITS(TRY)
@@ -29,6 +27,7 @@ const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) 
     }
     fixed = false;
     if (mode == FOLD_LINE) return nullptr;
+    if (mode == FOLD_PERSIST) return fold_any_persist();
     if (mode == FOLD_STEP) return fold_any_step(strided);
     return strided ? fold_any_misc_s() : fold_any_misc_c();
 }
@@ -63,6 +62,26 @@ cudaError_t fold_launch_line(const FoldArgs& a, int64_t nsteps, const FoldLaunch
     const void* k = fold_kernel(a.ax, false, FOLD_LINE, fixed);
     void* args[] = {(void*)&a, (void*)&nsteps};
     return cudaLaunchKernel(k, dim3(1), dim3(g.threads), args, g.smem, st);
+}
+
+FoldPersist fold_persist(const FoldAxis& x, bool many, int PS, int PC) {
+    FoldPersist p{};
+    FoldAxis y = x;
+    y.P = 2;
+    if (many) p.kernel = fold_kernel(y, false, FOLD_PERSIST, p.fixed);
+    if (many && p.fixed) {
+        p.PS = PS;
+        p.PC = PC;
+    } else {
+        y.P = 1;
+        p.kernel = fold_kernel(y, false, FOLD_PERSIST, p.fixed);
+        p.PS = 2;
+        p.PC = 1;
+    }
+    const int NR = x.R / 2 + 1, nk = x.A * x.B / 2 + 1, m = NR * (x.A > x.B ? x.A : x.B);
+    const int P = p.PS > p.PC ? p.PS : p.PC;
+    p.threads = p.fixed ? ((m > nk ? m : nk) * P + 31) / 32 * 32 : fold::kAnyThreads;
+    return p;
 }
 
 cudaError_t fold_set_smem(const FoldAxis& x, bool strided, int bytes) {

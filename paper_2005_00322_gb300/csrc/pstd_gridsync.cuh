@@ -47,13 +47,17 @@ __device__ __forceinline__ int ld_acquire_i(const int* p) {
 }
 
 // Barrier of all CTAs of the launch; false if a bounded wait gave up (here or
-// in another CTA).  All threads of every CTA must call it.
-__device__ bool grid_sync(const GridSync& g) {
+// in another CTA).  All threads of every CTA must call it.  `gen` is the
+// generation before the launch's first barrier, read by thread 0 and counted
+// on here: a read of it at each barrier is one more L2 round trip of a run's
+// chain.
+__device__ bool grid_sync(const GridSync& g, unsigned& gen) {
     __shared__ int ok;
     __syncthreads();
+    if (g.expected == 1) return true;     // one CTA and no arrival withheld
     if (threadIdx.x == 0) {
         ok = 1;
-        const unsigned my_gen = ld_acquire(g.gen);
+        const unsigned my_gen = gen++;
         __threadfence();
         const unsigned arrived = atomicAdd(g.count, 1u) + 1u;
         if (arrived == g.expected) {
@@ -75,6 +79,11 @@ __device__ bool grid_sync(const GridSync& g) {
     }
     __syncthreads();
     return ok != 0;
+}
+// (a launch counts on its own)
+__device__ bool grid_sync(const GridSync& g) {
+    unsigned gen = threadIdx.x == 0 && g.expected > 1 ? ld_acquire(g.gen) : 0;
+    return grid_sync(g, gen);
 }
 #endif
 

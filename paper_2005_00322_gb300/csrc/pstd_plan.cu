@@ -270,6 +270,7 @@ struct pstd_plan_s {
     int members = 1;                  // plans of the batch this one belongs to, whose passes share the GPU
     int persist_ok = 0;
     WLaunch pgeo{};
+    unsigned ptables = 0;             // FoldPersistArgs::tables
     cudaStream_t stream = nullptr;
     int ndim = 0;
     int64_t shape[4][3] = {};
@@ -760,10 +761,7 @@ int build_fold(pstd_plan_s* P, int i, const pstd::FoldChoice& ch, int os) {
     x.inner = a.inner;
     a.strided = a.inner > 1;
     x.wide = (int64_t)(a.N + 1) * a.inner >= (int64_t)1 << 30;
-    auto tiles = [&](int p) -> int64_t {
-        if (!a.strided) return (a.nlines + 2 * p - 1) / (2 * p);
-        return (a.nlines / a.inner) * ((a.inner + 2 * p - 1) / (2 * p));
-    };
+    auto tiles = [&](int p) { return pstd::fold_tiles(x, a.strided, p); };
     auto fits = [&](int p) {
         x.P = p;
         return pstd::fold::smem_bytes(x, a.strided) <= 200 * 1024;
@@ -828,10 +826,7 @@ int build_conv(pstd_plan_s* P, int i, const pstd::FoldChoice& ch) {
     x.nlines = a.nlines;
     x.inner = a.inner;
     a.strided = a.inner > 1;
-    auto tiles = [&](int p) -> int64_t {
-        if (!a.strided) return (a.nlines + 2 * p - 1) / (2 * p);
-        return (a.nlines / a.inner) * ((a.inner + 2 * p - 1) / (2 * p));
-    };
+    auto tiles = [&](int p) { return pstd::fold_tiles(x, a.strided, p); };
     // rows of 8 words where that still fills the GPU, 4 words else
     x.P = !a.strided ? 1 : (tiles(4) * P->members >= 2 * P->nsm ? 4 : 2);
     x.lgP = x.P == 4 ? 2 : (x.P == 2 ? 1 : 0);
@@ -1817,6 +1812,36 @@ int pstd_internal_launch_steps(pstd_plan_t* P, float* p, float* const* u, int64_
     return PSTD_OK;
 }
 
+// Pass of axis a in a cooperative run on kernel k, its work items and shared memory.
+static FoldArgs fold_persist_pass(pstd_plan_s* P, int a, const pstd::FoldPersist& k, float* p, float* const* u,
+                                  unsigned& items, size_t& smem) {
+    const Axis& A = P->ax[a];
+    FoldArgs f = fold_step(P, a, p, u);
+    if (k.fixed) {
+        f.ax.P = A.strided ? k.PS : k.PC;
+        f.ax.lgP = 0;
+        while ((1 << f.ax.lgP) < f.ax.P) ++f.ax.lgP;
+    }
+    items = (unsigned)pstd::fold_tiles(f.ax, A.strided, f.ax.P);
+    smem = pstd::fold::smem_bytes(f.ax, A.strided);
+    return f;
+}
+// The cooperative kernel of plans whose axes share a schedule: a compiled one
+// unless an axis needs 64-bit offsets, for many lines where every axis has them.
+static pstd::FoldPersist fold_persist_kernel(pstd_plan_s* const* plans, int n) {
+    FoldAxis x = plans[0]->ax[0].fax;
+    pstd::FoldChoice ch{};
+    pstd::fold_choose(x.L, ch);
+    bool many = ch.PS > 0;
+    for (int m = 0; m < n; ++m)
+        for (int a = 0; a < plans[m]->ndim; ++a) {
+            const Axis& A = plans[m]->ax[a];
+            x.wide |= A.fax.wide;
+            many = many && A.fax.P == (A.strided ? ch.PS : ch.PC);
+        }
+    return pstd::fold_persist(x, many, ch.PS, ch.PC);
+}
+
 // Barrier of a cooperative run on the words count, generation, status at `d`.
 static GridSync grid_barrier(unsigned* d, unsigned grid, unsigned withhold, long long spin_limit) {
     GridSync s;
@@ -1893,7 +1918,8 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
     int npass = 0;
     for (int m = 0; m < n; ++m) npass = plans[m]->ndim > npass ? plans[m]->ndim : npass;
     const bool fold = kind == 1 && plans[0]->ax[0].fold();
-    int fold_threads = 0;
+    pstd::FoldPersist fk{};
+    if (fold) fk = fold_persist_kernel(plans, n);
     const size_t esz = fold ? sizeof(FoldArgs) : (kind == 1 ? sizeof(WStep) : sizeof(StepArgs));
     S->h_args.assign((size_t)n * 3 * esz, 0);
     S->h_prefix.assign((size_t)3 * (n + 1), 0);
@@ -1909,11 +1935,12 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
                 Axis& A = P->ax[a];
                 unsigned char* slot = S->h_args.data() + ((size_t)m * 3 + k) * esz;
                 if (fold) {
-                    const FoldArgs f = fold_step(P, a, p[m], u + 3 * m);
+                    unsigned tiles;
+                    size_t sm;
+                    const FoldArgs f = fold_persist_pass(P, a, fk, p[m], u + 3 * m, tiles, sm);
                     std::memcpy(slot, &f, sizeof f);
-                    items = A.fgeo.grid;
-                    smem = A.fgeo.smem > smem ? A.fgeo.smem : smem;
-                    fold_threads = A.fgeo.threads > fold_threads ? A.fgeo.threads : fold_threads;
+                    items = tiles;
+                    smem = sm > smem ? sm : smem;
                 } else if (kind == 1) {
                     WStep w;
                     w.ax = A.wax;
@@ -1960,10 +1987,8 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const Axis& A0 = plans[0]->ax[0];
-    if (fold) {
-        if (fold_threads > pstd::fold::kAnyThreads) fold_threads = pstd::fold::kAnyThreads;
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pstd::fold_any_persist(), fold_threads, smem));
-    } else if (kind == 1) CK(wpersist_blocks(A0.L, A0.wv, A0.wgeo.threads, smem, &per_sm));
+    if (fold) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fk.kernel, fk.threads, smem));
+    else if (kind == 1) CK(wpersist_blocks(A0.L, A0.wv, A0.wgeo.threads, smem, &per_sm));
     else {
         CK(pstd::set_max_smem((int)smem));
         CK(pstd::k_step_persist_blocks(smem, &per_sm));
@@ -1982,8 +2007,7 @@ int pstd_internal_batch_persist_run(pstd_batch_persist_s** state, pstd_plan_t* c
         pa.mem = (const FoldArgs*)S->d_args;
         pa.prefix = S->d_prefix;
         void* args[] = {(void*)&pa};
-        CK(cudaLaunchCooperativeKernel(pstd::fold_any_persist(), dim3((unsigned)grid), dim3(fold_threads), args, smem,
-                                       st));
+        CK(cudaLaunchCooperativeKernel(fk.kernel, dim3((unsigned)grid), dim3(fk.threads), args, smem, st));
     } else if (kind == 1) {
         PersistArgs pa{};
         pa.ndim = npass;
@@ -2171,21 +2195,44 @@ int make_plan(const pstd_desc* desc, void* stream, const pstd_plan_opts* opts, i
             size_t smem = 0;
             int64_t items = 0;
             int threads = 0;
+            pstd::FoldPersist fk{};
+            if (fold) {
+                fk = fold_persist_kernel(&P, 1);
+                threads = fk.threads;
+            }
             for (int i = 0; i < P->ndim; ++i) {
-                const size_t sm = fold ? P->ax[i].fgeo.smem : P->ax[i].wgeo.smem;
-                const int64_t it = fold ? P->ax[i].fgeo.grid : P->ax[i].wgeo.grid;
-                const int th = fold ? P->ax[i].fgeo.threads : P->ax[i].wgeo.threads;
+                size_t sm = P->ax[i].wgeo.smem;
+                int64_t it = P->ax[i].wgeo.grid;
+                if (fold) {
+                    float* const none[3] = {};
+                    unsigned tiles;
+                    fold_persist_pass(P, i, fk, nullptr, none, tiles, sm);
+                    it = tiles;
+                } else {
+                    threads = P->ax[i].wgeo.threads > threads ? P->ax[i].wgeo.threads : threads;
+                }
                 smem = sm > smem ? sm : smem;
                 items = it > items ? it : items;
-                threads = th > threads ? th : threads;
             }
-            if (fold && threads > pstd::fold::kAnyThreads) threads = pstd::fold::kAnyThreads;
+            if (fold) {
+                // the tables of all axes beside the pass' buffer while no more than
+                // the default limit is needed
+                size_t tab = 0;
+                for (int i = 0; i < P->ndim; ++i) {
+                    const FoldAxis& x = P->ax[i].fax;
+                    tab += ((size_t)x.M + (size_t)x.R / 2 * x.nk + 2 * (x.N + 1)) * sizeof(float2);
+                }
+                smem = (smem + 15) / 16 * 16;
+                if (smem + tab <= 46 * 1024) {
+                    P->ptables = (unsigned)smem;
+                    smem += tab;
+                }
+            }
             int per_sm = 0, dev = 0, nsm = 0;
             cudaError_t e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
             if (e == cudaSuccess)
-                e = fold ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pstd::fold_any_persist(), threads,
-                                                                         smem)
+                e = fold ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fk.kernel, threads, smem)
                          : wpersist_blocks(P->ax[0].L, P->ax[0].wv, threads, smem, &per_sm);
             if (e == cudaSuccess) e = cudaMalloc((void**)&P->d_sync, 4 * sizeof(unsigned));
             if (e == cudaSuccess) e = cudaMemset(P->d_sync, 0, 4 * sizeof(unsigned));
@@ -2326,18 +2373,17 @@ int run_steps(pstd_plan_t* P, float* p, float* const* u, int64_t nsteps) {
         FoldPersistArgs pa{};
         pa.ndim = P->ndim;
         pa.nsteps = nsteps;
-        for (int a = 0; a < P->ndim; ++a) {
-            pa.ax[a] = fold_step(P, a, p, u);
-            pa.strided[a] = P->ax[a].strided ? 1 : 0;
-            pa.items[a] = P->ax[a].fgeo.grid;
-        }
+        pa.tables = P->ptables;
+        const pstd::FoldPersist fk = fold_persist_kernel(&P, 1);
+        size_t smem;
+        for (int a = 0; a < P->ndim; ++a) pa.ax[a] = fold_persist_pass(P, a, fk, p, u, pa.items[a], smem);
         pa.sync = grid_barrier(P->d_sync, P->pgeo.grid,
                                (unsigned)(P->opts.withhold_arrivals > 0 ? P->opts.withhold_arrivals : 0),
                                P->opts.spin_limit);
         CK(cudaMemsetAsync(P->d_sync, 0, sizeof(unsigned), P->stream));   // arrival count
         void* args[] = {(void*)&pa};
-        CK(cudaLaunchCooperativeKernel(pstd::fold_any_persist(), dim3(P->pgeo.grid), dim3(P->pgeo.threads), args,
-                                       P->pgeo.smem, P->stream));
+        CK(cudaLaunchCooperativeKernel(fk.kernel, dim3(P->pgeo.grid), dim3(P->pgeo.threads), args, P->pgeo.smem,
+                                       P->stream));
         P->last_launches = 1;
         return PSTD_OK;
     }
