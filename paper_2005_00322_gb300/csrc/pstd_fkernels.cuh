@@ -184,19 +184,24 @@ __global__ void __launch_bounds__(persist_threads<CS, CC>(), persist_blocks<CS, 
 }  // namespace fold
 
 // Lengths 2^k and 3 2^k: those that had kernels of every kind on the register
-// FFTs.  Their cooperative run has a form for many lines too (the form for few, 2
-// and 1 pairs, took 807 us per 256^3 step and 145 per 128^3 step).
+// FFTs.  Their derivatives and velocity conversions are compiled (256^3: 61 to 65
+// us a pass, 115 to 120 on run-time radices, 84 to 133 on the register FFTs; on
+// other lengths the run-time radices stand against the shared-memory program:
+// 200 x 180 x 150 47 to 57 against 111 to 136), and their cooperative run has a form
+// for many lines too (the form for few, 2 and 1 pairs, took 807 us per 256^3 step
+// and 145 per 128^3 step).
 constexpr bool fold_dyadic(int L) {
     while (L % 2 == 0) L /= 2;
     return L == 1 || L == 3;
 }
-// Kernel of a schedule (mode FOLD_STEP, FOLD_ORDER2, FOLD_LINE or FOLD_PERSIST)
+// Kernel of a schedule (any mode but FOLD_CONV)
 // with P pairs per CTA, or null where it is not compiled; one function per
 // translation unit.
 template <class C, bool STR>
 const void* fold_mode(int mode) {
     if (mode == FOLD_STEP) return (const void*)fold::k_fold<C, STR, FOLD_STEP>;
     if (mode == FOLD_ORDER2) return (const void*)fold::k_fold<C, STR, FOLD_ORDER2>;
+    if constexpr (fold_dyadic(C::R * C::A * C::B)) return (const void*)fold::k_fold<C, STR, FOLD_MISC>;
     return nullptr;
 }
 template <int R, int A, int B, int PS, int PC>

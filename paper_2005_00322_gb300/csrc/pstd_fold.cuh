@@ -74,7 +74,8 @@ struct FoldAxis {
 enum { FOLD_STEP = 0, FOLD_GRAD_P = 1, FOLD_GRAD_U = 2, FOLD_TO_SPEC = 3, FOLD_FROM_SPEC = 4, FOLD_ORDER2 = 5,
        FOLD_CONV = 7,        // leapfrog pass of an embedded line: p -> u, u += , u -> p, p +=
        // kernels that loop over FOLD_STEP passes: a 1-D run, a cooperative run
-       FOLD_LINE = 6, FOLD_PERSIST = 8 };
+       FOLD_LINE = 6, FOLD_PERSIST = 8,
+       FOLD_MISC = -2 };     // kernels for GRAD_P, GRAD_U, TO_SPEC or FROM_SPEC, chosen at run time (-1: for any mode)
 
 struct FoldArgs {
     FoldAxis ax;
@@ -356,7 +357,7 @@ PSTD_HD float ldc(const float* p) {
 // runs of 2P words, straight between memory and registers); otherwise
 // contiguous lines, read in place (the R residues share their sectors in L1)
 // and written through rows in shared memory.  MODE < 0: the mode is a
-// run-time value.  Byte offsets from a CTA-uniform base are 32-bit in the fixed
+// run-time value (FOLD_MISC: of four).  Byte offsets from a CTA-uniform base are 32-bit in the fixed
 // schedules (the plan takes the run-time form for fields beyond 4 GiB): with
 // 64-bit ones the address arithmetic cost more than the FFT (40 integer against
 // 36 floating-point instructions per point on 256^3).
@@ -403,9 +404,14 @@ struct Pass {
     PSTD_HD bool in_half() const { return mode<PM>() == FOLD_GRAD_U || mode<PM>() == FOLD_TO_SPEC; }
     template <int PM = MODE>
     PSTD_HD bool out_half() const { return mode<PM>() == FOLD_GRAD_P || mode<PM>() == FOLD_FROM_SPEC; }
+    // (constant false in FOLD_MISC kernels)
+    template <int PM = MODE>
+    PSTD_HD bool stepping() const { if constexpr (MODE == FOLD_MISC) return false; else return mode<PM>() == FOLD_STEP; }
+    template <int PM = MODE>
+    PSTD_HD bool order2() const { if constexpr (MODE == FOLD_MISC) return false; else return mode<PM>() == FOLD_ORDER2; }
     PSTD_HD bool conv() const {
         if constexpr (MODE == FOLD_CONV) return true;
-        else if constexpr (MODE >= 0) return false;
+        else if constexpr (MODE != -1) return false;
         else return a.ax.cN > 0;
     }
     PSTD_HD int nhalf() const { return conv() ? a.ax.cN : N(); }     // stored half-nodes
@@ -685,7 +691,7 @@ struct Pass {
                     if (in_half<PM>()) half_twiddle<r_, false>(w, std::make_integer_sequence<int, r_>{});
                 }
                 // spectral update; outputs q >= R/2 hold sg x (canonical bin)
-                if (mode<PM>() == FOLD_STEP) {
+                if (stepping<PM>()) {
                     const Slots sl = slots(p, k, nv == 2 * P());
                     if constexpr (!ahead_u) {
                         // all slots are read before any is written (bins of a
@@ -719,7 +725,7 @@ struct Pass {
                     for (int q = 0; q < r_; ++q) {
                         // the signs of the canonical bin's two uses cancel
                         const float f = ldc(&(MODE == FOLD_CONV && PM == FOLD_GRAD_U ? a.f2 : a.f)[bin(k, q)]);
-                        w[q] = mode<PM>() == FOLD_ORDER2 ? cscale(w[q], f)
+                        w[q] = order2<PM>() ? cscale(w[q], f)
                                                      : make_float2(-rmul(f, w[q].y), rmul(f, w[q].x));
                     }
                 }
@@ -967,13 +973,13 @@ struct Pass {
     PSTD_HD void emit(float* y, bool ok, float c) const {
         if (!ok) return;
         const int64_t off = y - a.out;
-        if (mode() == FOLD_STEP || mode() == FOLD_CONV) {
+        if (stepping() || mode() == FOLD_CONV) {
             *y = radd(a.acc_in[off], c);
             return;
         }
         const float v = a.accumulate ? radd(*y, c) : c;
         *y = v;
-        if (mode() == FOLD_ORDER2 && a.pout) a.pout[off] = radd(a.in[off], v);
+        if (order2() && a.pout) a.pout[off] = radd(a.in[off], v);
     }
     // contiguous lines from their rows
     PSTD_HD void finish() {
@@ -988,7 +994,7 @@ struct Pass {
                 for (int i = lane; i < len; i += 32, q += 36, z += 32) {
                     if constexpr (ahead) {
                         *z = *q;
-                        if (mode() == FOLD_ORDER2 && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
+                        if (order2() && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
                     } else emit(z, true, *q);
                 }
             }

@@ -19,7 +19,7 @@ const void* fold_kernel(const FoldAxis& x, bool strided, int mode, bool& fixed) 
 #undef TRY
         return nullptr;
     }
-    if (!x.wide && (mode == FOLD_STEP || mode == FOLD_ORDER2 || mode == FOLD_LINE || mode == FOLD_PERSIST)) {
+    if (!x.wide && !x.cN) {
 #define TRY(U) \
     if (const void* k = fold_unit_##U(x.R, x.A, x.B, x.P, strided, mode)) return k;
         PSTD_FOLD_UNITS(TRY)
