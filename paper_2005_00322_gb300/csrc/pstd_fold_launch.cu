@@ -42,13 +42,13 @@ cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cu
     cfg.blockDim = dim3(fixed || g.threads < fold::kAnyThreads ? g.threads : fold::kAnyThreads);
     cfg.dynamicSmemBytes = g.smem;
     cfg.stream = st;
-    // passes of a step follow one another: a pass may start (and fetch its
-    // tables) while the previous one drains; it waits before touching fields
+    // passes follow one another: a pass may start (and fetch its tables) while the
+    // previous one drains; it waits before touching fields
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = !overlap ? 0 : a.mode == FOLD_STEP || a.mode == FOLD_ORDER2 || a.mode == FOLD_CONV ? 1 : 0;
+    cfg.numAttrs = overlap ? 1 : 0;
     void* args[] = {(void*)&a};
     return cudaLaunchKernelExC(&cfg, k, args);
 }
