@@ -864,6 +864,24 @@ struct Pass {
                 by_full([&](auto full) {
                     const bool la = full || va(p), lb = full || vb(p);
                     const OutOff oo = out_off(p, j0, half);
+                    // what the outputs are added to, requested before the first store
+                    // (which may alias it: one load after another took 9 us of a
+                    // 512^2 half-step start)
+                    constexpr bool add = STR && !ahead;
+                    float2 old[add ? a_ : 1];
+                    if constexpr (add) {
+                        if (const float* za = added(ya)) {
+                            const float* zb = za + line_step(nout());
+#pragma unroll
+                            for (int e = 0; e < a_; ++e) {
+                                int i;
+                                bool mir;
+                                const bool ok = out_index<a_>(e, self, j0 + R() * B() * e, half, i, mir);
+                                const Off off = oo.at(e, mir);
+                                old[e] = make_float2(ok && la ? ld(za, off) : 0.0f, ok && lb ? ld(zb, off) : 0.0f);
+                            }
+                        }
+                    }
 #pragma unroll
                     for (int e = 0; e < a_; ++e) {
                         int i;
@@ -884,8 +902,8 @@ struct Pass {
                                     }
                                 }
                             } else {
-                                emit(ya + off / 4, ok && la, rmul(sgn, x[e].x));
-                                emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y));
+                                emit(ya + off / 4, ok && la, rmul(sgn, x[e].x), old[e].x);
+                                emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y), old[e].y);
                             }
                         } else {
                             // row position of node (lo + i) or half-node i
@@ -969,17 +987,20 @@ struct Pass {
                 for (int i = lane; i < len; i += 32) y[l * (int64_t)len + i] = st[l * pitch + row_word(i)];
         }
     }
-    // *y = its new value from contribution c
-    PSTD_HD void emit(float* y, bool ok, float c) const {
+    // what contributions to `y`, in a.out, are added to; null: nothing
+    PSTD_HD const float* added(const float* y) const {
+        if (stepping() || mode() == FOLD_CONV) return a.acc_in + (y - a.out);
+        return a.accumulate ? y : nullptr;
+    }
+    // *y = its new value from contribution c and the value it is added to
+    PSTD_HD void emit(float* y, bool ok, float c, float old) const {
         if (!ok) return;
-        const int64_t off = y - a.out;
-        if (stepping() || mode() == FOLD_CONV) {
-            *y = radd(a.acc_in[off], c);
-            return;
-        }
-        const float v = a.accumulate ? radd(*y, c) : c;
+        const float v = stepping() || mode() == FOLD_CONV || a.accumulate ? radd(old, c) : c;
         *y = v;
-        if (order2() && a.pout) a.pout[off] = radd(a.in[off], v);
+        if (order2() && a.pout) {
+            const int64_t off = y - a.out;
+            a.pout[off] = radd(a.in[off], v);
+        }
     }
     // contiguous lines from their rows
     PSTD_HD void finish() {
@@ -991,11 +1012,22 @@ struct Pass {
             for (int l = wid; l < nv; l += nw) {
                 const float* q = st + l * pitch + row_word(lane + lo);   // + 36 words per 32 positions
                 float* z = y + l * (int64_t)len + lane;
-                for (int i = lane; i < len; i += 32, q += 36, z += 32) {
-                    if constexpr (ahead) {
+                if constexpr (ahead) {
+                    for (int i = lane; i < len; i += 32, q += 36, z += 32) {
                         *z = *q;
                         if (order2() && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
-                    } else emit(z, true, *q);
+                    }
+                } else {
+                    // (four at a time: loads before stores, as in p5)
+                    const float* o = added(z);
+                    for (int i = lane; i < len; i += 128, q += 144, z += 128) {
+                        float old[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) old[k] = o && i + 32 * k < len ? o[i - lane + 32 * k] : 0.0f;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (i + 32 * k < len) emit(z + 32 * k, true, q[36 * k], old[k]);
+                    }
                 }
             }
         }
