@@ -162,13 +162,13 @@ struct Axis {
     // folded passes (pstd_fold.cuh; wv == kFold, wl: lanes per pair)
     FoldAxis fax{};
     FoldLaunch fgeo{};
-    float2* d_ftab = nullptr;         // twiddles tw | tc | th
-    float2* d_fcoef = nullptr;        // step coefficients per bin
-    float* d_fgrad[OP_COUNT] = {};    // derivative multipliers per bin (GRAD_P, GRAD_U, INIT_P)
+    float* d_ftab = nullptr;                // all of its tables (upload_fold), and into it:
+    const float2* d_fcoef = nullptr;        // step coefficients per bin
+    const float* d_fgrad[OP_COUNT] = {};    // derivative multipliers per bin (GRAD_P, GRAD_U, INIT_P)
     float* d_f2fold = nullptr;        // second-order multiplier per bin, on first use
     bool fold() const { return wl > 0 && wv == kFold; }
     bool cfold = false;               // convolution passes on folded transforms (fax; wl == 0)
-    float* d_fconv[2] = {nullptr, nullptr};   // step multipliers p -> u, u -> p
+    const float* d_fconv[2] = {nullptr, nullptr};   // step multipliers p -> u, u -> p (in d_ftab)
     // BF16 three-way split form on tcgen05: the two operators' BF16 slices
     // (D1: N x lp, D2: lp x N) and their TMA tensor maps
     uint16_t* d_tc16[2] = {nullptr, nullptr};
@@ -749,6 +749,28 @@ int build_order2(pstd_plan_s* P, int i) {
     return PSTD_OK;
 }
 
+// All tables of an axis' folded passes as one allocation and one copy: the
+// twiddles, `cf` (float2), then the lists `f`, which start at *at.
+int upload_fold(Axis& a, const pstd::FoldTables& t, const std::vector<float2>& cf,
+                std::initializer_list<const std::vector<float>*> f, const float** at) {
+    std::vector<float> all;
+    for (const auto* v : {&t.tw, &t.tc, &t.th, &cf})
+        for (const float2& c : *v) {
+            all.push_back(c.x);
+            all.push_back(c.y);
+        }
+    const size_t n2 = all.size();
+    for (const auto* v : f) all.insert(all.end(), v->begin(), v->end());
+    const int rc = upload(all, &a.d_ftab);
+    if (rc != PSTD_OK) return rc;
+    FoldAxis& x = a.fax;
+    x.tw = (const float2*)a.d_ftab;
+    x.tc = x.tw + t.tw.size();
+    x.th = x.tc + t.tc.size();
+    *at = a.d_ftab + n2;
+    return PSTD_OK;
+}
+
 // Folded passes of axis i (pstd_fold.cuh): geometry, tables and launch.  `os`
 // line pairs per CTA (-1: chosen here).
 int build_fold(pstd_plan_s* P, int i, const pstd::FoldChoice& ch, int os) {
@@ -793,24 +815,17 @@ int build_fold(pstd_plan_s* P, int i, const pstd::FoldChoice& ch, int os) {
     a.fgeo.grid = (unsigned)tiles(p);
     a.fgeo.threads = pstd::fold_threads(x);
     a.fgeo.smem = pstd::fold::smem_bytes(x, a.strided);
-    std::vector<float2> tab(t.tw);
-    tab.insert(tab.end(), t.tc.begin(), t.tc.end());
-    tab.insert(tab.end(), t.th.begin(), t.th.end());
-    int rc;
-    if ((rc = upload(tab, &a.d_ftab)) != PSTD_OK) return rc;
-    x.tw = a.d_ftab;
-    x.tc = x.tw + t.tw.size();
-    x.th = x.tc + t.tc.size();
     std::vector<float2> cf;
     pstd::fold_step_coef(x, a.dx, -d.dt / d.rho0, -d.dt * d.rho0 * d.c0 * d.c0, cf);
-    if ((rc = upload(cf, &a.d_fcoef)) != PSTD_OK) return rc;
-    const struct { int op; double scale; } g[3] = {
-        {OP_GRAD_P, 1.0}, {OP_GRAD_U, 1.0}, {OP_INIT_P, d.dt / (2.0 * d.rho0)}};
-    for (const auto& q : g) {
-        std::vector<float> f;
-        pstd::fold_grad_coef(x, a.dx, q.scale, f);
-        if ((rc = upload(f, &a.d_fgrad[q.op])) != PSTD_OK) return rc;
-    }
+    std::vector<float> f[3];
+    pstd::fold_grad_coef(x, a.dx, 1.0, f[0]);
+    pstd::fold_grad_coef(x, a.dx, d.dt / (2.0 * d.rho0), f[1]);
+    const float* at;
+    const int rc = upload_fold(a, t, cf, {&f[0], &f[1]}, &at);
+    if (rc != PSTD_OK) return rc;
+    a.d_fcoef = x.th + t.th.size();
+    a.d_fgrad[OP_GRAD_P] = a.d_fgrad[OP_GRAD_U] = at;
+    a.d_fgrad[OP_INIT_P] = at + f[0].size();
     a.wl = pstd::fold_lanes(x);
     a.wv = kFold;
     return PSTD_OK;
@@ -833,23 +848,20 @@ int build_conv(pstd_plan_s* P, int i, const pstd::FoldChoice& ch) {
     a.fgeo.grid = (unsigned)tiles(x.P);
     a.fgeo.threads = pstd::fold_threads(x);
     a.fgeo.smem = pstd::fold::smem_bytes(x, a.strided);
-    std::vector<float2> tab(t.tw);
-    tab.insert(tab.end(), t.tc.begin(), t.tc.end());
-    tab.insert(tab.end(), t.th.begin(), t.th.end());
-    int rc;
-    if ((rc = upload(tab, &a.d_ftab)) != PSTD_OK) return rc;
-    x.tw = a.d_ftab;
-    x.tc = x.tw + t.tw.size();
-    x.th = x.tc + t.tc.size();
     const std::vector<double> f1 = pstd::conv_coef(x, a.group2, a.dx, host_fft);
-    const struct { float** d; double scale; } out[5] = {
-        {&a.d_fconv[0], -d.dt / d.rho0}, {&a.d_fconv[1], -d.dt * d.rho0 * d.c0 * d.c0},
-        {&a.d_fgrad[OP_GRAD_P], 1.0}, {&a.d_fgrad[OP_GRAD_U], 1.0}, {&a.d_fgrad[OP_INIT_P], d.dt / (2.0 * d.rho0)}};
-    for (const auto& o : out) {
-        std::vector<float> f(f1.size());
-        for (size_t b = 0; b < f.size(); ++b) f[b] = (float)(f1[b] * o.scale);
-        if ((rc = upload(f, o.d)) != PSTD_OK) return rc;
+    const double scale[4] = {-d.dt / d.rho0, -d.dt * d.rho0 * d.c0 * d.c0, 1.0, d.dt / (2.0 * d.rho0)};
+    std::vector<float> f[4];
+    for (int o = 0; o < 4; ++o) {
+        f[o].resize(f1.size());
+        for (size_t b = 0; b < f1.size(); ++b) f[o][b] = (float)(f1[b] * scale[o]);
     }
+    const float* at;
+    const int rc = upload_fold(a, t, {}, {&f[0], &f[1], &f[2], &f[3]}, &at);
+    if (rc != PSTD_OK) return rc;
+    a.d_fconv[0] = at;
+    a.d_fconv[1] = at + f1.size();
+    a.d_fgrad[OP_GRAD_P] = a.d_fgrad[OP_GRAD_U] = at + 2 * f1.size();
+    a.d_fgrad[OP_INIT_P] = at + 3 * f1.size();
     a.cfold = true;
     return PSTD_OK;
 }
@@ -1282,11 +1294,7 @@ void free_plan_memory(pstd_plan_s* P) {
         cudaFree(a.d_ph);
         cudaFree(a.d_tc);
         cudaFree(a.d_ftab);
-        cudaFree(a.d_fcoef);
         cudaFree(a.d_f2fold);
-        cudaFree(a.d_fconv[0]);
-        cudaFree(a.d_fconv[1]);
-        for (float* f : a.d_fgrad) cudaFree(f);
         cudaFree(a.d_f2);
         cudaFree(a.d_dense2);
         for (int o = 0; o < 2; ++o)
