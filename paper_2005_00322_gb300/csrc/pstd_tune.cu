@@ -114,6 +114,14 @@ extern "C" int pstd_plan_autotune(const pstd_desc* desc, void* stream, const pst
         if (cudaMalloc((void**)&f[i], bytes) != cudaSuccess || cudaMemset(f[i], 0, bytes) != cudaSuccess)
             rc = PSTD_ENOMEM;
     }
+    // lines of axis a are contiguous where the later axes store one node
+    bool strided[3] = {};
+    int64_t stored[3] = {1, 1, 1}, inner = 1;
+    pstd_field_shape(P0, 0, stored);
+    for (int a = desc->ndim - 1; a >= 0; --a) {
+        strided[a] = inner > 1;
+        inner *= stored[a];
+    }
     pstd_free(P0);
     cudaStream_t st = (cudaStream_t)stream;
     Tuned best{o, -1.0, -1.0};
@@ -126,8 +134,7 @@ extern "C" int pstd_plan_autotune(const pstd_desc* desc, void* stream, const pst
         // the compiled pairs per CTA of the folded passes
         pstd::FoldChoice ch{};
         if (desc->bc[a][0] != PSTD_PERIODIC && L >= 16 && pstd::fold_choose(L, ch) && ch.PS > 0) {
-            const bool strided = a + 1 < desc->ndim;
-            for (int sq : {strided ? ch.PS : ch.PC, strided ? 2 : 1}) {
+            for (int sq : {strided[a] ? ch.PS : ch.PC, strided[a] ? 2 : 1}) {
                 pstd_plan_opts c = best.opts;
                 c.variant[a] = 6;
                 c.seqs_per_cta[a] = sq;

@@ -87,3 +87,18 @@ def test_batch(cooperative):
     for (n, w), (p0, u0), (p, _) in zip(GRIDS, host, fields):
         assert rel(p, oracle(n, w, time_step(n), p0, u0, STEPS).p) < 1e-4, n
     b.close()
+
+
+def test_autotuned():
+    """The candidates of a contiguous axis before the last: its compiled pairs."""
+    from paper_2005_00322_gb300 import Solver
+    ncells, bcs = (48, 48, 2), [("N", "D"), ("D", "D"), ("D", "D")]
+    s = Solver(ncells, DX, bcs, dt=time_step(ncells), autotune=True)
+    variant, _, pairs, _ = s.schedule()[1]
+    assert variant != 6 or pairs in (1, 8)
+    p0, u0 = start(s.shapes)
+    p, us = on_gpu(p0, u0)
+    s.run(p, us, STEPS)
+    s.sync()
+    assert rel(p, oracle(ncells, bcs, time_step(ncells), p0, u0, STEPS).p) < 1e-4
+    s.close()
