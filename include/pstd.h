@@ -234,7 +234,11 @@ int pstd_step(pstd_plan_t* plan, float* p, float* const* u);
 /* `nsteps` >= 0 leapfrog steps in place.  The plan records one block of
  * steps in a CUDA graph per (p, u) pointer set on first use and replays it;
  * a tail shorter than the block is launched directly.  A 1-D run on a
- * compiled folded schedule is one kernel that loops over its steps.
+ * compiled folded schedule is one kernel that loops over its steps.  The first
+ * run of a block or more on a 2-D plan of at most 2 M points, both axes on
+ * compiled folded schedules, allocates two more fields of the pressure shape,
+ * a stream and two events, which the plan keeps (both axis passes of a step
+ * then run side by side; without them, one after the other).
  * Errors: PSTD_EINVAL, PSTD_ECUDA. */
 int pstd_run(pstd_plan_t* plan, float* p, float* const* u, int64_t nsteps);
 

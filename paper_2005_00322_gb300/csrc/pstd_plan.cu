@@ -1284,6 +1284,19 @@ int build_axis(pstd_plan_s* P, int i) {
     return PSTD_OK;
 }
 
+void free_side(pstd_plan_s* P) {
+    for (float*& c : P->d_C) {
+        cudaFree(c);
+        c = nullptr;
+    }
+    for (auto& e : P->ev) {
+        if (e) cudaEventDestroy(e);
+        e = nullptr;
+    }
+    if (P->side) cudaStreamDestroy(P->side);
+    P->side = nullptr;
+}
+
 void free_plan_memory(pstd_plan_s* P) {
     for (auto& a : P->ax) {
         cudaFree(a.d_tw);
@@ -1311,10 +1324,7 @@ void free_plan_memory(pstd_plan_s* P) {
         }
     }
     cudaFree(P->d_S);
-    for (float* c : P->d_C) cudaFree(c);
-    for (auto e : P->ev)
-        if (e) cudaEventDestroy(e);
-    if (P->side) cudaStreamDestroy(P->side);
+    free_side(P);
     cudaFree(P->d_energy);
     for (auto* b : P->d_pad) cudaFree(b);
     cudaFree(P->d_Spad);
@@ -1681,6 +1691,9 @@ int launch_order2_step(pstd_plan_s* P, float* p, float* q, int64_t* launches) {
 // ends with p += C.  512^2: 9.5 us per step one pass after the other.
 bool side_by_side(pstd_plan_s* P) {
     if (P->side_ok >= 0) return P->side_ok == 1;
+    // (a stream that is being captured decides nothing: nothing can be allocated)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(P->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
     P->side_ok = 0;
     bool ok = P->ndim == 2 && P->opts.form == 0 && P->stream != nullptr && !P->persist_ok;
     for (int a = 0; a < 2 && ok; ++a) {
@@ -1691,14 +1704,18 @@ bool side_by_side(pstd_plan_s* P) {
     // beyond 2 M points the passes fill the GPU by themselves
     const int64_t n = P->shape[0][0] * P->shape[0][1];
     if (!ok || n > (int64_t)2 << 20) return false;
-    for (auto& c : P->d_C)
-        if (cudaMalloc((void**)&c, (size_t)n * sizeof(float)) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-    if (cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking) != cudaSuccess) return false;
-    for (auto& e : P->ev)
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
+    // allowed beside another thread's capture
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    for (auto& c : P->d_C) ok = ok && cudaMalloc((void**)&c, (size_t)n * sizeof(float)) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking) == cudaSuccess;
+    for (auto& e : P->ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!ok) {
+        cudaGetLastError();
+        free_side(P);
+        return false;
+    }
     P->side_ok = 1;
     return true;
 }
