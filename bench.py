@@ -68,10 +68,10 @@ def cells(w) -> int:
 
 def csrc_digest() -> str:
     """Digest of the sources that build and launch the axis-pass kernels
-    (the register-FFT passes and the plan that schedules them)."""
+    (the folded and register-FFT passes and the plan that schedules them)."""
     h = hashlib.sha256()
     for f in sorted(os.listdir(CSRC)):
-        if f.startswith("pstd_w") or f in ("pstd_plan.cu", "pstd_internal.h", "pstd_ops.cuh"):
+        if f.startswith(("pstd_w", "pstd_f")) or f in ("pstd_plan.cu", "pstd_internal.h", "pstd_ops.cuh"):
             h.update(open(os.path.join(CSRC, f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -654,10 +654,10 @@ def main():
     achieved = alg_bytes / per_launch / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "kernel": ("k_wgrad dir 4 (second-order axis pass)" if args.form == "order2"
+                "kernel": ("k_fold (second-order axis pass)" if args.form == "order2"
                            else "k_fold (fused axis pass)") if single
-                else "every member's axis passes (k_wstep register passes, k_step generic / convolution "
-                     "passes), concurrent graph branches",
+                else "every member's axis passes (k_fold, folded and folded-convolution passes; k_fold_any), "
+                     "concurrent graph branches",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks else "fallback 6.8 TB/s",
                 "alg_bytes_per_launch": alg_bytes,
                 "launch_s": per_launch if single else None, "step_s": step_s}

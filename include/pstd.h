@@ -142,7 +142,9 @@ int pstd_plan(const pstd_desc* desc, void* stream, pstd_plan_t** out);
  * the symmetry-folded line (one half of the extension and of its spectrum);
  * without options the register-FFT variants serve periodic axes and lengths
  * below 16.  An unavailable variant gives PSTD_EINVAL.
- * seqs_per_cta: line pairs per CTA (a power of two). */
+ * seqs_per_cta: line pairs per CTA (a power of two).  Set with variant -1 it
+ * selects the register-FFT schedule where the length has one (the folded
+ * passes, faster on walled axes, take it with variant 6). */
 typedef struct {
     int variant[3];
     int seqs_per_cta[3];
@@ -166,7 +168,8 @@ typedef struct {
     int form;
     /* 1: pstd_run is one cooperative kernel for all its steps, the CTAs
      * meeting at a bounded-wait grid barrier between axis passes (when every
-     * axis runs the same register-FFT schedule; otherwise ignored).  A wait
+     * axis has the same length and folded or register-FFT schedule; otherwise
+     * ignored).  A wait
      * that exceeds spin_limit polls (0: about a second) ends the kernel and
      * pstd_sync returns PSTD_ETIMEOUT. */
     int persistent;
@@ -390,23 +393,24 @@ int64_t pstd_batch_last_launch_count(const pstd_batch_t* batch);
  * axis passes, last axis first, are split into work items (line groups or
  * tiles) over all members, which the resident CTAs take in turn, meeting at a
  * software grid barrier between passes.  When every axis of every member has
- * the same register-FFT schedule (e.g. the 4^d wall combinations of one
- * grid) the kernel runs those passes, with each member's velocity conversion
- * before and after it; otherwise every axis runs the generic shared-memory
- * program (its own FFT, convolution or dense route).  Each barrier wait is
+ * the same length and folded or register-FFT schedule (e.g. the 4^d wall
+ * combinations of one cube) the kernel runs those passes, with each member's
+ * velocity conversion before and after it; otherwise every axis runs the
+ * generic shared-memory program (its own FFT, convolution or dense route; the
+ * first such run allocates the convolution's tables).  Each barrier wait is
  * bounded by spin_limit polls (0: a default of about a second); on giving up
  * the kernel ends and pstd_batch_sync reports PSTD_ETIMEOUT.
  * withhold_arrivals > 0 makes every barrier wait for that many arrivals that
  * never come (to test the bounded wait).  Results equal the graph path's bit
- * for bit on the register-FFT kernel and on members whose axes all take the
- * generic program there too; a register-FFT axis run by the generic program
- * agrees to rounding.  Errors: PSTD_EINVAL; PSTD_EUNSUPPORTED for a
+ * for bit on the folded and register-FFT kernels and on members whose axes all
+ * take the generic program there too; a folded, folded-convolution or
+ * register-FFT axis run by the generic program agrees to rounding.  Errors: PSTD_EINVAL; PSTD_EUNSUPPORTED for a
  * dense-operator form (pstd_plan_opts.form != 0 is not set by pstd_batch_plan,
  * so this does not arise for its members). */
 int pstd_batch_set_persistent(pstd_batch_t* batch, int enable, long long spin_limit, int withhold_arrivals);
 
-/* The cooperative kernel pstd_batch_set_persistent would use: 1 register-FFT
- * passes, 2 the generic program.  Errors: PSTD_EINVAL. */
+/* The cooperative kernel pstd_batch_set_persistent would use: 1 folded or
+ * register-FFT passes, 2 the generic program.  Errors: PSTD_EINVAL. */
 int pstd_batch_persistent_kind(const pstd_batch_t* batch);
 
 /* Wait for the batch's stream.  PSTD_ETIMEOUT (reported once) if a barrier

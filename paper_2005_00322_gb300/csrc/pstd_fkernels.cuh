@@ -1,8 +1,8 @@
 // pstd_fkernels.cuh -- kernels of the folded passes (pstd_fold.cuh).
 //
 // Two forms share one source: radices and line pairs per CTA fixed at compile
-// time (Cfg, the lengths of the power-of-two and 3 x 2^k grids), or read from
-// the plan (AnyCfg, every other length with a schedule).  pstd_fold_*.cu
+// time (Cfg, the lengths of pstd_fold_list.h), or read from the plan (AnyCfg,
+// every other length with a schedule).  pstd_fold_*.cu
 // instantiate them; fold_kernel finds the one of a schedule.
 #pragma once
 
@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(cfg_threads<C>()) k_fold_line(const __grid_con
 }
 // Run-time radices: every phase holds a switch over them, so registers are those
 // of the largest (it spills above radix 10) and offsets are 64-bit; about three
-// times slower per point than fixed radices (224^3 477 us per step), still twice
-// as fast as the routes these lengths had (112 x 70: 57 -> 22 us).
+// times slower per point than fixed radices (224^3 376 us per step), still twice
+// as fast as the routes these lengths had (112 x 70: 57 -> 20 us).
 template <bool STR, int MODE>
 __global__ void __launch_bounds__(kAnyThreads, 2) k_fold_any(const __grid_constant__ FoldArgs a) {
     extern __shared__ float4 wsm4[];

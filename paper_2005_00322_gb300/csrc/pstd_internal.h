@@ -28,8 +28,8 @@ int pstd_internal_cuda_fail(cudaError_t e, const char* what);
 
 // A batch of plans as one cooperative kernel per run (pstd_batch_set_persistent).
 struct pstd_batch_persist_s;
-// Which cooperative kernel the plans allow: 1 the register-FFT passes (every
-// axis of every member on one register schedule; the velocities are in their
+// Which cooperative kernel the plans allow: 1 folded or register-FFT passes (every
+// axis of every member on one schedule; the velocities are in their
 // spectrum form around the run, as for pstd_internal_launch_steps), 2 the
 // generic CTA program on every axis (velocities as stored), 0 none (a
 // dense-operator form).

@@ -1130,7 +1130,9 @@ int build_axis(pstd_plan_s* P, int i) {
 
     if (a.kind == 2 && (rc = build_conv_tables(P, i)) != PSTD_OK) return rc;
 
-    // register-FFT passes where a schedule exists.  Measured on GB300 (512^2,
+    // Register-FFT passes where a schedule exists: periodic axes, lengths below
+    // 16, and walled ones whose caller asks for a variant or (the rules for V = 3, 4,
+    // 5 below) for pairs per CTA alone.  Measured on GB300 (512^2,
     // 256^3, 384^3): the latency schedules (8 or 12 elements per lane) beat
     // the throughput ones wherever they exist, with 2 line pairs per CTA once
     // the axis has enough lines to keep 2 CTAs per SM busy.
