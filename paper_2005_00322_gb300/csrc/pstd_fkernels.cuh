@@ -75,15 +75,15 @@ __global__ void __launch_bounds__(cfg_threads<C>()) k_fold_line(const __grid_con
 #ifdef __CUDA_ARCH__
     extern __shared__ float4 wsm4[];
     for (int64_t s = 0; s < nsteps; ++s) {
-        fold_pass<C, false, FOLD_STEP>(a, 0, wsm4, threadIdx.x, blockDim.x);
+        fold_pass<OntoP<C>, false, FOLD_STEP>(a, 0, wsm4, threadIdx.x, blockDim.x);
         __syncthreads();
     }
 #endif
 }
 // Run-time radices: every phase holds a switch over them, so registers are those
 // of the largest (it spills above radix 10) and offsets are 64-bit; about three
-// times slower per point than fixed radices (224^3 376 us per step), still twice
-// as fast as the routes these lengths had (112 x 70: 57 -> 20 us).
+// times slower per point than fixed radices (224^3 442 us per step), still twice
+// as fast as the routes these lengths had (112 x 70: 57 -> 22 us).
 template <bool STR, int MODE>
 __global__ void __launch_bounds__(kAnyThreads, 2) k_fold_any(const __grid_constant__ FoldArgs a) {
     extern __shared__ float4 wsm4[];

@@ -267,8 +267,14 @@ struct Cfg {
     static constexpr int R = R_, A = A_, B = B_, P = P_;
     static constexpr bool fixed = R_ > 0;
     static constexpr bool resident = false;
+    static constexpr bool onto_p_only = false;
 };
 using AnyCfg = Cfg<0, 0, 0, 0>;
+// contiguous step passes of a last axis alone: acc_in == in
+template <class C>
+struct OntoP : C {
+    static constexpr bool onto_p_only = true;
+};
 // tables that may lie in shared memory (a cooperative run's)
 template <class C>
 struct Resident : C {
@@ -807,7 +813,7 @@ struct Pass {
             // (contiguous lines of an axis that is not the last -- the later axes
             // store one node -- add onto the accumulator like strided ones)
             if constexpr (onto_p) {
-                if (a.acc_in == a.in) return;
+                if (C::onto_p_only || a.acc_in == a.in) return;
             }
             by_full([&](auto full) {
                 const float* xa = base(MODE == FOLD_ORDER2 ? (const float*)a.out : a.acc_in, nout());
@@ -864,22 +870,19 @@ struct Pass {
                 by_full([&](auto full) {
                     const bool la = full || va(p), lb = full || vb(p);
                     const OutOff oo = out_off(p, j0, half);
-                    // what the outputs are added to, requested before the first store
-                    // (which may alias it: one load after another took 9 us of a
-                    // 512^2 half-step start)
-                    constexpr bool add = STR && !ahead;
-                    float2 old[add ? a_ : 1];
-                    if constexpr (add) {
-                        if (const float* za = added(ya)) {
-                            const float* zb = za + line_step(nout());
+                    // FOLD_MISC: the values that outputs are added to, requested before
+                    // the first store (which may alias them: one load after another
+                    // took 9 us of a 512^2 half-step start)
+                    constexpr bool early = STR && MODE == FOLD_MISC;
+                    float2 old[early ? a_ : 1];
+                    if constexpr (early) {
 #pragma unroll
-                            for (int e = 0; e < a_; ++e) {
-                                int i;
-                                bool mir;
-                                const bool ok = out_index<a_>(e, self, j0 + R() * B() * e, half, i, mir);
-                                const Off off = oo.at(e, mir);
-                                old[e] = make_float2(ok && la ? ld(za, off) : 0.0f, ok && lb ? ld(zb, off) : 0.0f);
-                            }
+                        for (int e = 0; e < a_; ++e) {
+                            int i;
+                            bool mir;
+                            const bool ok = a.accumulate && out_index<a_>(e, self, j0 + R() * B() * e, half, i, mir);
+                            const Off off = oo.at(e, mir);
+                            old[e] = make_float2(ok && la ? ld(ya, off) : 0.0f, ok && lb ? ld(yb, off) : 0.0f);
                         }
                     }
 #pragma unroll
@@ -901,9 +904,13 @@ struct Pass {
                                         if (ok && lb) put(qa + line_step(nout()), off, radd(pk[e].y, v.y));
                                     }
                                 }
+                            } else if constexpr (early) {
+                                const float2 c = make_float2(rmul(sgn, x[e].x), rmul(sgn, x[e].y));
+                                if (ok && la) put(ya, off, a.accumulate ? radd(old[e].x, c.x) : c.x);
+                                if (ok && lb) put(yb, off, a.accumulate ? radd(old[e].y, c.y) : c.y);
                             } else {
-                                emit(ya + off / 4, ok && la, rmul(sgn, x[e].x), old[e].x);
-                                emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y), old[e].y);
+                                emit(ya + off / 4, ok && la, rmul(sgn, x[e].x));
+                                emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y));
                             }
                         } else {
                             // row position of node (lo + i) or half-node i
@@ -987,20 +994,17 @@ struct Pass {
                 for (int i = lane; i < len; i += 32) y[l * (int64_t)len + i] = st[l * pitch + row_word(i)];
         }
     }
-    // what contributions to `y`, in a.out, are added to; null: nothing
-    PSTD_HD const float* added(const float* y) const {
-        if (stepping() || mode() == FOLD_CONV) return a.acc_in + (y - a.out);
-        return a.accumulate ? y : nullptr;
-    }
-    // *y = its new value from contribution c and the value it is added to
-    PSTD_HD void emit(float* y, bool ok, float c, float old) const {
+    // *y = its new value from contribution c
+    PSTD_HD void emit(float* y, bool ok, float c) const {
         if (!ok) return;
-        const float v = stepping() || mode() == FOLD_CONV || a.accumulate ? radd(old, c) : c;
-        *y = v;
-        if (order2() && a.pout) {
-            const int64_t off = y - a.out;
-            a.pout[off] = radd(a.in[off], v);
+        const int64_t off = y - a.out;
+        if (mode() == FOLD_STEP || mode() == FOLD_CONV) {
+            *y = radd(a.acc_in[off], c);
+            return;
         }
+        const float v = a.accumulate ? radd(*y, c) : c;
+        *y = v;
+        if (mode() == FOLD_ORDER2 && a.pout) a.pout[off] = radd(a.in[off], v);
     }
     // contiguous lines from their rows
     PSTD_HD void finish() {
@@ -1012,22 +1016,24 @@ struct Pass {
             for (int l = wid; l < nv; l += nw) {
                 const float* q = st + l * pitch + row_word(lane + lo);   // + 36 words per 32 positions
                 float* z = y + l * (int64_t)len + lane;
-                if constexpr (ahead) {
-                    for (int i = lane; i < len; i += 32, q += 36, z += 32) {
-                        *z = *q;
-                        if (order2() && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
-                    }
-                } else {
+                int i = lane;
+                if constexpr (MODE == FOLD_MISC) {
                     // (four at a time: loads before stores, as in p5)
-                    const float* o = added(z);
-                    for (int i = lane; i < len; i += 128, q += 144, z += 128) {
+                    for (; i + 96 < len; i += 128, q += 144, z += 128) {
                         float old[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) old[k] = o && i + 32 * k < len ? o[i - lane + 32 * k] : 0.0f;
+                        for (int k = 0; k < 4; ++k) old[k] = a.accumulate ? z[32 * k] : 0.0f;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (i + 32 * k < len) emit(z + 32 * k, true, q[36 * k], old[k]);
+                        for (int k = 0; k < 4; ++k) z[32 * k] = a.accumulate ? radd(old[k], q[36 * k]) : q[36 * k];
                     }
+                }
+                for (; i < len; i += 32, q += 36, z += 32) {
+                    if constexpr (ahead) {
+                        *z = *q;
+                        if (mode() == FOLD_ORDER2 && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
+                    } else if constexpr (MODE == FOLD_MISC) {
+                        *z = a.accumulate ? radd(*z, *q) : *q;
+                    } else emit(z, true, *q);
                 }
             }
         }
