@@ -870,19 +870,23 @@ struct Pass {
                 by_full([&](auto full) {
                     const bool la = full || va(p), lb = full || vb(p);
                     const OutOff oo = out_off(p, j0, half);
-                    // FOLD_MISC: the values that outputs are added to, requested before
-                    // the first store (which may alias them: one load after another
-                    // took 9 us of a 512^2 half-step start)
-                    constexpr bool early = STR && MODE == FOLD_MISC;
+                    // Derivatives and the like: the values that outputs are added to,
+                    // requested before the first store (which may alias them: one load
+                    // after another took 9 us of a 512^2 half-step start).  Run-time
+                    // radices above 8 have no registers for it, nor has their step.
+                    constexpr bool early = STR && MODE < 0 && (C::fixed || a_ <= 8);
                     float2 old[early ? a_ : 1];
                     if constexpr (early) {
+                        if (const float* za = added(ya)) {
+                            const float* zb = za + line_step(nout());
 #pragma unroll
-                        for (int e = 0; e < a_; ++e) {
-                            int i;
-                            bool mir;
-                            const bool ok = a.accumulate && out_index<a_>(e, self, j0 + R() * B() * e, half, i, mir);
-                            const Off off = oo.at(e, mir);
-                            old[e] = make_float2(ok && la ? ld(ya, off) : 0.0f, ok && lb ? ld(yb, off) : 0.0f);
+                            for (int e = 0; e < a_; ++e) {
+                                int i;
+                                bool mir;
+                                const bool ok = out_index<a_>(e, self, j0 + R() * B() * e, half, i, mir);
+                                const Off off = oo.at(e, mir);
+                                old[e] = make_float2(ok && la ? ld(za, off) : 0.0f, ok && lb ? ld(zb, off) : 0.0f);
+                            }
                         }
                     }
 #pragma unroll
@@ -905,9 +909,8 @@ struct Pass {
                                     }
                                 }
                             } else if constexpr (early) {
-                                const float2 c = make_float2(rmul(sgn, x[e].x), rmul(sgn, x[e].y));
-                                if (ok && la) put(ya, off, a.accumulate ? radd(old[e].x, c.x) : c.x);
-                                if (ok && lb) put(yb, off, a.accumulate ? radd(old[e].y, c.y) : c.y);
+                                emit(ya + off / 4, ok && la, rmul(sgn, x[e].x), old[e].x);
+                                emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y), old[e].y);
                             } else {
                                 emit(ya + off / 4, ok && la, rmul(sgn, x[e].x));
                                 emit(yb + off / 4, ok && lb, rmul(sgn, x[e].y));
@@ -998,13 +1001,28 @@ struct Pass {
     PSTD_HD void emit(float* y, bool ok, float c) const {
         if (!ok) return;
         const int64_t off = y - a.out;
-        if (mode() == FOLD_STEP || mode() == FOLD_CONV) {
+        if (stepping() || mode() == FOLD_CONV) {
             *y = radd(a.acc_in[off], c);
             return;
         }
         const float v = a.accumulate ? radd(*y, c) : c;
         *y = v;
-        if (mode() == FOLD_ORDER2 && a.pout) a.pout[off] = radd(a.in[off], v);
+        if (order2() && a.pout) a.pout[off] = radd(a.in[off], v);
+    }
+    // what contributions to `y`, in a.out, are added to; null: nothing
+    PSTD_HD const float* added(const float* y) const {
+        if (stepping() || mode() == FOLD_CONV) return a.acc_in + (y - a.out);
+        return a.accumulate ? y : nullptr;
+    }
+    // the same with that value at hand
+    PSTD_HD void emit(float* y, bool ok, float c, float old) const {
+        if (!ok) return;
+        const float v = stepping() || mode() == FOLD_CONV || a.accumulate ? radd(old, c) : c;
+        *y = v;
+        if (order2() && a.pout) {
+            const int64_t off = y - a.out;
+            a.pout[off] = radd(a.in[off], v);
+        }
     }
     // contiguous lines from their rows
     PSTD_HD void finish() {
@@ -1017,22 +1035,21 @@ struct Pass {
                 const float* q = st + l * pitch + row_word(lane + lo);   // + 36 words per 32 positions
                 float* z = y + l * (int64_t)len + lane;
                 int i = lane;
-                if constexpr (MODE == FOLD_MISC) {
+                if constexpr (MODE < 0) {
                     // (four at a time: loads before stores, as in p5)
+                    const float* o = added(z);
                     for (; i + 96 < len; i += 128, q += 144, z += 128) {
                         float old[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) old[k] = a.accumulate ? z[32 * k] : 0.0f;
+                        for (int k = 0; k < 4; ++k) old[k] = o ? o[i - lane + 32 * k] : 0.0f;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) z[32 * k] = a.accumulate ? radd(old[k], q[36 * k]) : q[36 * k];
+                        for (int k = 0; k < 4; ++k) emit(z + 32 * k, true, q[36 * k], old[k]);
                     }
                 }
                 for (; i < len; i += 32, q += 36, z += 32) {
                     if constexpr (ahead) {
                         *z = *q;
                         if (mode() == FOLD_ORDER2 && a.pout) a.pout[z - a.out] = radd(a.in[z - a.out], *q);
-                    } else if constexpr (MODE == FOLD_MISC) {
-                        *z = a.accumulate ? radd(*z, *q) : *q;
                     } else emit(z, true, *q);
                 }
             }

@@ -44,7 +44,8 @@ cudaError_t fold_launch(const FoldArgs& a, bool strided, const FoldLaunch& g, cu
     cfg.stream = st;
     // passes and conversions follow one another: one may start (and fetch its tables)
     // while the previous one drains; it waits before touching fields.  A derivative
-    // is mostly a call of its own, which the attribute makes 0.8 us longer.
+    // is mostly a call of its own with nothing to overlap (512^2 half-step start: 26 us
+    // with the attribute and without).
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
