@@ -15,8 +15,10 @@
 // is taken: idle lanes count a third (a 128^3 step takes 39.0 us with (4, 8, 8),
 // whose phases have 24, 24 and 33 items, 41.7 with (8, 4, 8) and its 40, 20 and 17;
 // 48^3 7.9 with (6, 4, 4), 9.4 with (8, 3, 4); 810 x 810 x 32 437 with (12, 9, 15), 505
-// with (18, 9, 10); the runner-up is faster on 150^3, 69 against 73 us, and by 3 or 4
-// percent on the planes of 24, 30, 150 and 320 cells).  R above 10 costs a tenth more (p3 is the longest
+// with (18, 9, 10); 320^2 is the one grid measured where the runner-up is faster, 6.0
+// against 6.2 us).  R = 10 competes only where no smaller R stays within 48 lanes:
+// at 150 and 180 cells it would cost planes 4 to 10 percent (180 x 512 6.6 us, 6.0 with
+// (8, 5, 9)).  R above 10 costs a tenth more (p3 is the longest
 // serial phase: a 512^2 step takes 9.5 us with (8, 8, 16), 10.2 with (16, 8, 8)), any
 // radix above 10 a fifth more and above 16 twice that (registers).  PS = 8 makes
 // each global access of a strided pass a run of 16 words (256^3: 254 us per step
@@ -71,7 +73,7 @@
 #define PSTD_FOLD_U5(X) \
     X(4, 3, 4, 8, 8) \
     X(6, 5, 6, 8, 4) \
-    X(10, 6, 6, 8, 4) \
+    X(8, 5, 9, 8, 4) \
     X(10, 5, 9, 4, 4) \
     X(8, 10, 12, 4, 2) \
     X(8, 8, 16, 4, 2) \
@@ -87,7 +89,7 @@
 #define PSTD_FOLD_U7(X) \
     X(4, 3, 5, 8, 8) \
     X(6, 6, 6, 8, 4) \
-    X(10, 5, 6, 8, 4) \
+    X(6, 5, 10, 8, 4) \
     X(6, 8, 10, 8, 4) \
     X(8, 9, 12, 4, 2) \
     X(8, 10, 16, 4, 2) \

@@ -33,8 +33,11 @@ def cost(R, A, B):
 
 def by_rule(L):
     inner = [1, 2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16]
-    R, A, B = min(((R, A, L // R // A) for R in range(2, 21, 2) if L % R == 0 for A in inner
-                   if L // R % A == 0 and L // R // A in inner), key=lambda s: cost(*s))
+    every = [(R, A, L // R // A) for R in range(2, 21, 2) if L % R == 0 for A in inner
+             if L // R % A == 0 and L // R // A in inner]
+    if any(s[0] < 10 and lanes(*s) <= 48 for s in every):
+        every = [s for s in every if s[0] != 10]
+    R, A, B = min(every, key=lambda s: cost(*s))
     n = lanes(R, A, B)
     return R, A, B, 8 if n <= 48 else 4, 8 if n <= 20 else 4 if n < 60 else 2
 
